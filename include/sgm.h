@@ -236,16 +236,19 @@ int sgm_batch_autotune(sgm_batch b, const uint8_t *const *left, const uint8_t *c
 int sgm_batch_device_bytes(sgm_batch b, size_t *bytes);
 
 /* Shape of the aggregation kernel of later calls on h (the paper has no
- * counterpart): resident 4-warp blocks per SM (1..16) and 8-disparity chunks
- * per lane: 1, 2 or 4 for every direction, or SGM_AGG_CHUNKS_MIXED (the
- * long-axis scanlines, rows when W >= H, at 1 and the other directions at 2).
+ * counterpart): resident 4-warp blocks per SM (1..16; no more blocks are
+ * launched than there is work for) and disparities per lane, counted in chunks
+ * of 8: 1 (the default), 2 or 4, or SGM_AGG_CHUNKS_MIXED.  With 1 a lane holds
+ * one chunk, or half of one on the long-axis scanlines (rows when W >= H) while
+ * D <= 128, whose chain of steps sets the kernel's duration; with 2 and 4 it
+ * holds that many chunks in every direction; MIXED is one chunk on the
+ * long-axis scanlines and two in the other directions.
  * SGM_ERR_UNSUPPORTED above what D allows (D must span at least that many
- * chunks; the 16-bit costs of SGM_COST_SAD take 1).  With c chunks per lane a
- * scanline's D disparities occupy D / (8 c) lanes (rounded up to a power of
- * two), so a warp walks more scanlines at once with fewer instructions per
+ * chunks; the 16-bit costs of SGM_COST_SAD take 1).  More disparities per lane
+ * let a warp walk more scanlines at once with fewer instructions per
  * disparity estimate, but each step of a scanline takes longer.  Results do
- * not depend on either setting.  A new handle starts with 3 blocks per SM and
- * 1 chunk per lane, or with what sgm_autotune chose for its shape. */
+ * not depend on either setting.  A new handle starts with 4 blocks per SM and
+ * setting 1, or with what sgm_autotune chose for its shape. */
 #define SGM_AGG_CHUNKS_MIXED 3
 int sgm_set_aggregation(sgm_handle h, int blocks_per_sm, int chunks_per_lane);
 int sgm_get_aggregation(sgm_handle h, int *blocks_per_sm, int *chunks_per_lane);

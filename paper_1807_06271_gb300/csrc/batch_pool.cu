@@ -129,11 +129,9 @@ int layout_groups(sgm_batch_s *b, int ng, bool upload, size_t at, size_t *end) {
             t.planes = b->pool + ps.planes;
             t.W = ps.W;
             t.H = ps.H;
-            t.D = ps.D;
-            t.lps = lanes_per_scanline(ps.D) / b->cpl;
-            t.ragged = ps.D != 8 * lanes_per_scanline(ps.D);
+            t.Dp = ps.Dp;
             t.nplanes = b->npaths;
-            t.jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->cpl);
+            t.jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl);
             prefix[k + 1] = prefix[k] + t.jobs.nlong;
             prefix[np + 1 + k + 1] = prefix[np + 1 + k] + (t.jobs.jbegin[t.jobs.n] - t.jobs.nlong);
         }
@@ -211,7 +209,7 @@ int enqueue(sgm_batch_s *b, const uint8_t *const *left, const uint8_t *const *ri
             // (overlapped) dependency on the one before it.
             const int i = g.pairs[0];
             PairSlot &ps = b->pairs[i];
-            const PathJobs jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->cpl);
+            const PathJobs jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl);
             if (costs(i, job_state) != cudaSuccess ||
                 launch_aggregate(b->pool + ps.cost, ps.W, ps.H, ps.D, b->p.P1, b->p.P2, b->wide != 0, jobs,
                                  b->pool + ps.planes, b->npaths, job_state, b->blocks_per_sm, b->cpl,
@@ -228,7 +226,7 @@ int enqueue(sgm_batch_s *b, const uint8_t *const *left, const uint8_t *const *ri
                 cudaStreamWaitEvent(g.stream, ps.ready, 0) != cudaSuccess)
                 return SGM_ERR_CUDA;
         }
-        if (cudaMemsetAsync(job_state, 0, kJobStateBytes, g.stream) != cudaSuccess ||
+        if (cudaMemsetAsync(job_state, 0, sizeof(unsigned), g.stream) != cudaSuccess ||
             launch_aggregate_batch(reinterpret_cast<const BatchAggPair *>(b->pool + g.table), (int)g.pairs.size(),
                                    reinterpret_cast<const int *>(b->pool + g.prefix), b->p.P1, b->p.P2, b->wide != 0,
                                    b->cpl, job_state, b->blocks_per_sm, g.stream) != cudaSuccess ||

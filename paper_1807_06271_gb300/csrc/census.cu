@@ -142,14 +142,15 @@ __global__ void __launch_bounds__(kBX *kBY)
 
 // ---------------------------------------------------------------------------
 // Matching cost volume (Eq. 1): C(x,y,d) = popc(code_l(x,y) ^ code_r(x-d,y)),
-// or the code width when x-d < 0, for d < D; padding slots d >= D hold the
-// code width too.  One CTA per segment of kSeg pixels of one row: the
+// or the code width when x-d < 0, for d < D; padding slots d >= D hold
+// kPadCost.  One CTA per segment of kSeg pixels of one row: the
 // segment's left codes and the right codes it reaches (kSeg + Dp + 2 of them)
-// are staged in shared memory.  A thread computes one DPL-disparity chunk of
-// two neighbouring pixels from DPL + 1 consecutive right codes read as
+// are staged in shared memory.  A thread computes two words (eight
+// disparities, four at either end of the range) of the folded records of
+// two neighbouring pixels from two runs of five right codes read as
 // aligned vectors, with consecutive threads on consecutive pixel pairs
 // (conflict-free reads); the segment is transposed through a padded shared
-// tile and written out with coalesced DPL-byte stores (the segment's Dp-byte
+// tile and written out with coalesced 8-byte stores (the segment's Dp-byte
 // pixel records are contiguous in global memory).  popc runs on the XU pipe
 // (16 per SM per clock; two per estimate for 64-bit codes), which bounds
 // this kernel.
@@ -163,32 +164,14 @@ constexpr int kCostThreads = 64, kSeg = 32;
 __device__ __forceinline__ uint32_t popcnt(uint32_t v) { return __popc(v); }
 __device__ __forceinline__ uint32_t popcnt(uint64_t v) { return __popcll(v); }
 
-// Bytes of one chunk word: word w of a lane holds disparities 2w, 2w+1, 2w+h, 2w+1+h
-// (h = DPL/2) in its bytes 0..3, the order in which the aggregation unpacks them.
-template <int DPL>
-__device__ __forceinline__ void pack_chunk(const uint32_t (&c)[DPL], uint32_t (&w)[DPL / 4]) {
-    constexpr int h = DPL / 2;
-#pragma unroll
-    for (int i = 0; i < DPL / 4; i++)
-        w[i] = (c[2 * i + 1 + h] * 256u + c[2 * i + h]) * 65536u + (c[2 * i + 1] * 256u + c[2 * i]);
-}
-
-template <int DPL>
-__device__ __forceinline__ void st_shared_chunk(uint8_t *p, const uint32_t (&w)[DPL / 4]) {
-    if constexpr (DPL == 8) *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
-    else *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-template <typename CodeT, int DPL, bool RAGGED>
+template <typename CodeT, bool RAGGED>
 __global__ void __launch_bounds__(kCostThreads)
     cost_kernel(const CodeT *__restrict__ codes, int W, int H, int D, int Dp, int nbits,
                 uint8_t *__restrict__ cost, unsigned *__restrict__ job_state) {
     wait_for_predecessor();
-    if (job_state && blockIdx.x == 0 && blockIdx.y == 0)
-        for (int i = threadIdx.x; i < (int)(kJobStateBytes / sizeof(unsigned)); i += kCostThreads) job_state[i] = 0u;
-    using VecT = typename std::conditional<DPL == 8, uint2, uint4>::type;
+    if (job_state && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *job_state = 0u;
     extern __shared__ __align__(16) unsigned char cost_smem[];
-    const int stride = Dp + DPL;  // padded tile row (bytes)
+    const int stride = Dp + 8;  // padded tile row (bytes)
     uint8_t *tile = cost_smem;                                          // [kSeg][stride]
     const int tile_bytes = (kSeg * stride + 15) & ~15;
     CodeT *cl = reinterpret_cast<CodeT *>(cost_smem + tile_bytes);     // [kSeg]
@@ -204,76 +187,77 @@ __global__ void __launch_bounds__(kCostThreads)
         cr[i] = (xr >= 0 && xr < W && in_range((long long)W * H + (long long)y * W + xr, 2LL * W * H)) ? rowr[xr] : 0;
     }
     __syncthreads();
-    const int chunks = Dp / DPL;
+    const int chunks = Dp / 8;
     const bool border = x0 < Dp;  // only the first segments see x - d < 0
-    // A thread takes one DPL-disparity chunk i of the pixel pair (px, px+1), px even.
-    // Column x - d of pixel px sits at cr[px - d + Dp + 1]: for the chunk's
-    // disparities DPL*i + j the pair needs the DPL + 1 codes w[k] = cr[s + k],
-    // s = px + Dp + 2 - DPL*(i + 1) (even, so the run is 16-byte aligned for
-    // 8-byte codes; 2 <= s and s + DPL <= kSeg + Dp): pixel px uses
-    // w[DPL - 1 - j], pixel px + 1 uses w[DPL - j].
-    // A thread's pixel pair is the same for all its chunks (kCostThreads is a
+    // A thread takes the two words (four pairs) i of the pixel pair (px, px+1), px
+    // even: the disparities 4i + e and Dp-1-4i-e, e < 4.  Column x - d of pixel px
+    // sits at cr[px - d + Dp + 1], so the pair needs two runs of five codes:
+    // wl[k] = cr[px + Dp - 2 - 4i + k] (pixel px uses wl[3 - e], px + 1 wl[4 - e]) and
+    // wh[k] = cr[px + 2 + 4i + k] (wh[e] and wh[e + 1]); both start at an even
+    // index, so the codes are read as aligned vectors of two.
+    // A thread's pixel pair is the same for all its words (kCostThreads is a
     // multiple of kSeg / 2), so its two left codes are read once.
     static_assert(kCostThreads % (kSeg / 2) == 0, "one pixel pair per thread");
     const int px = 2 * (threadIdx.x % (kSeg / 2));
+    auto two = [](const CodeT *p, CodeT &a, CodeT &b) {
+        if constexpr (sizeof(CodeT) == 8) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+            a = v.x;
+            b = v.y;
+        } else {
+            const uint2 v = *reinterpret_cast<const uint2 *>(p);
+            a = v.x;
+            b = v.y;
+        }
+    };
     CodeT a0, a1;
-    if constexpr (sizeof(CodeT) == 8) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(cl + px);
-        a0 = v.x;
-        a1 = v.y;
-    } else {
-        const uint2 v = *reinterpret_cast<const uint2 *>(cl + px);
-        a0 = v.x;
-        a1 = v.y;
-    }
+    two(cl + px, a0, a1);
     for (int it = threadIdx.x; it < (kSeg / 2) * chunks; it += kCostThreads) {
         const int i = it / (kSeg / 2);
-        const int sidx = px + Dp + 2 - DPL * (i + 1);
-        CodeT w[DPL + 1];
+        const CodeT *rl = cr + px + Dp - 2 - 4 * i, *rh = cr + px + 2 + 4 * i;
+        CodeT wl[5], wh[5];
+        two(rl, wl[0], wl[1]);
+        two(rl + 2, wl[2], wl[3]);
+        wl[4] = rl[4];
+        two(rh, wh[0], wh[1]);
+        two(rh + 2, wh[2], wh[3]);
+        wh[4] = rh[4];
 #pragma unroll
-        for (int k = 0; k < DPL / 2; k++) {
-            if constexpr (sizeof(CodeT) == 8) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(cr + sidx + 2 * k);
-                w[2 * k] = v.x;
-                w[2 * k + 1] = v.y;
-            } else {
-                const uint2 v = *reinterpret_cast<const uint2 *>(cr + sidx + 2 * k);
-                w[2 * k] = v.x;
-                w[2 * k + 1] = v.y;
+        for (int p = 0; p < 2; p++) {
+            const CodeT a = p ? a1 : a0;
+            uint32_t lo[4], hi[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                lo[e] = popcnt(a ^ wl[3 + p - e]);
+                hi[e] = popcnt(a ^ wh[p + e]);
             }
-        }
-        w[DPL] = cr[sidx + DPL];
-        uint32_t c[DPL], e[DPL];
+            if (RAGGED || border) {
+                const int x = x0 + px + p;
 #pragma unroll
-        for (int j = 0; j < DPL; j++) {
-            c[j] = popcnt(a0 ^ w[DPL - 1 - j]);
-            e[j] = popcnt(a1 ^ w[DPL - j]);
-        }
-        if (RAGGED || border) {
-            const int x = x0 + px;
-#pragma unroll
-            for (int j = 0; j < DPL; j++) {
-                const int d = DPL * i + j;
-                if ((RAGGED && d >= D) || x - d < 0) c[j] = (uint32_t)nbits;
-                if ((RAGGED && d >= D) || x + 1 - d < 0) e[j] = (uint32_t)nbits;
+                for (int e = 0; e < 4; e++) {
+                    const int dl = 4 * i + e, dh = Dp - 1 - dl;
+                    if (x - dl < 0) lo[e] = (uint32_t)nbits;
+                    if (x - dh < 0) hi[e] = (uint32_t)nbits;
+                    if (RAGGED && dl >= D) lo[e] = kPadCost;
+                    if (RAGGED && dh >= D) hi[e] = kPadCost;
+                }
             }
+            uint2 w;
+            w.x = (hi[0] * 256u + hi[1]) * 65536u + (lo[0] * 256u + lo[1]);
+            w.y = (hi[2] * 256u + hi[3]) * 65536u + (lo[2] * 256u + lo[3]);
+            *reinterpret_cast<uint2 *>(tile + (px + p) * stride + 8 * i) = w;
         }
-        uint32_t vc[DPL / 4], ve[DPL / 4];
-        pack_chunk<DPL>(c, vc);
-        pack_chunk<DPL>(e, ve);
-        st_shared_chunk<DPL>(tile + px * stride + DPL * i, vc);
-        st_shared_chunk<DPL>(tile + (px + 1) * stride + DPL * i, ve);
     }
     __syncthreads();
     const int npx = min(kSeg, W - x0);
     uint8_t *out = cost + ((size_t)y * W + x0) * Dp;
     for (int k = threadIdx.x; k < npx * chunks; k += kCostThreads) {
         const int px = k / chunks, q = k - px * chunks;
-        // a record of DPL bytes starting at byte o of the W x H x Dp volume
-        const long long o = ((long long)y * W + x0 + px) * Dp + DPL * q;
-        if (in_range(o, (long long)W * H * Dp - DPL + 1))
-            *reinterpret_cast<VecT *>(out + (size_t)px * Dp + DPL * q) =
-                *reinterpret_cast<const VecT *>(tile + px * stride + DPL * q);
+        // a record of 8 bytes starting at byte o of the W x H x Dp volume
+        const long long o = ((long long)y * W + x0 + px) * Dp + 8 * q;
+        if (in_range(o, (long long)W * H * Dp - 8 + 1))
+            *reinterpret_cast<uint2 *>(out + (size_t)px * Dp + 8 * q) =
+                *reinterpret_cast<const uint2 *>(tile + px * stride + 8 * q);
     }
 }
 
@@ -318,29 +302,24 @@ cudaError_t launch_cost(const void *codes, int code_bytes, int W, int H, int D, 
     if (kernel == SGM_COST_KERNEL_TENSOR_CORES)
         return launch_cost_mma(codes, code_bytes, W, H, D, nbits, cost, job_state, status, s);
     if (kernel != SGM_COST_KERNEL_CUDA_CORES) return cudaErrorInvalidValue;
-    const int Dp = padded_disparities(D), dpl = disparities_per_lane(D);
-    const size_t smem = (((size_t)kSeg * (Dp + dpl) + 15) & ~(size_t)15) + (size_t)(2 * kSeg + Dp + 2) * code_bytes;
+    const int Dp = padded_disparities(D);
+    const size_t smem = (((size_t)kSeg * (Dp + 8) + 15) & ~(size_t)15) + (size_t)(2 * kSeg + Dp + 2) * code_bytes;
     const dim3 grid((W + kSeg - 1) / kSeg, H);
-    cudaError_t e;
+    auto go = [&](auto kernel, auto *c) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        return launch_k(kernel, grid, dim3(kCostThreads), smem, s, c, W, H, D, Dp, nbits, cost, job_state);
+    };
     const bool rag = D != Dp;
-#define SGM_COST(T, P, R)                                                                                        \
-    do {                                                                                                         \
-        e = cudaFuncSetAttribute(cost_kernel<T, P, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-        if (e != cudaSuccess) return e;                                                                          \
-        e = launch_k(cost_kernel<T, P, R>, grid, dim3(kCostThreads), smem, s, (const T *)codes, W, H, D, Dp,   \
-                     nbits, cost, job_state);                                                                    \
-        if (e != cudaSuccess) return e;                                                                          \
-    } while (0)
-#define SGM_COST2(T, P)                \
-    do {                               \
-        if (rag) SGM_COST(T, P, true); \
-        else SGM_COST(T, P, false);    \
-    } while (0)
-    if (dpl != 8) return cudaErrorInvalidValue;
-    if (code_bytes == 4) SGM_COST2(uint32_t, 8);
-    else SGM_COST2(uint64_t, 8);
-#undef SGM_COST2
-#undef SGM_COST
+    cudaError_t e;
+    if (code_bytes == 4) {
+        const uint32_t *c = (const uint32_t *)codes;
+        e = rag ? go(cost_kernel<uint32_t, true>, c) : go(cost_kernel<uint32_t, false>, c);
+    } else {
+        const uint64_t *c = (const uint64_t *)codes;
+        e = rag ? go(cost_kernel<uint64_t, true>, c) : go(cost_kernel<uint64_t, false>, c);
+    }
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

@@ -46,7 +46,7 @@
 //   permute adds the fourth; the bytes go to the pixel's row of a tile T.
 //   Records: each thread then takes a quarter of one pixel's 8-disparity
 //   groups: it reads its window of T (word loads and one funnel shift, since
-//   the start differs per pixel), puts each group in the lane-chunk byte
+//   the start differs per pixel), puts each group in the folded
 //   order (two byte permutes) and writes it into the segment's records in a
 //   staging buffer; one cp.async.bulk copies the segment's contiguous records
 //   to the cost volume.  Slots with x - d < 0 or d >= D get nbits, as in the
@@ -194,8 +194,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     static_assert(DP == 32 || DP == 64 || DP == 128, "tensor-core cost kernel: Dp of 32, 64 or 128");
     extern __shared__ __align__(1024) unsigned char mma_smem[];
     wait_for_predecessor();
-    if (job_state && blockIdx.x == 0)
-        for (int i = threadIdx.x; i < (int)(kJobStateBytes / sizeof(unsigned)); i += kThreads) job_state[i] = 0u;
+    if (job_state && blockIdx.x == 0 && threadIdx.x == 0) *job_state = 0u;
     const int tid = threadIdx.x, warp = tid >> 5, t = tid & 31;
     const int segs_row = (W + kM - 1) / kM;
     const long long nseg = (long long)segs_row * H;
@@ -358,45 +357,45 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int y = s / segs_row, x0 = (s - y * segs_row) * kM;
         unsigned char *O = mma_smem + L::kO + (k & 1) * (kM * DP);
         {
-            // records: pixel i = 8 * warp + t / 4, chunks CPP * p .. CPP * p + CPP - 1, p = t % 4.
+            // records: pixel i = 8 * warp + t / 4, word pairs CPP * p .. CPP * p + CPP - 1, p = t % 4.
             // Pixel i (lane t_i = i % 32 of its quarter) reads bytes u = 0 .. DP-1 of its T row from
-            // t_i + 1 on, u <-> d = DP - 1 - u.  With word U[m] = bytes 4m .. 4m+3 of the part that
-            // starts at u = DP - 8 CPP (p + 1), chunk q = CPP p + m (d = 8q .. 8q+7) is
-            // U[2 CPP - 2 - 2m] (d = 8q+7 .. 8q+4) and the next word (d = 8q+3 .. 8q).
+            // t_i + 1 on, u <-> d = DP - 1 - u.  Word pair j holds the disparities 4j + e and DP-1-4j-e:
+            // the four bytes from u = DP - 4 - 4j (d = 4j+3 .. 4j) and those from u = 4j (d = DP-1-4j ..).
             const int i = 8 * warp + (t >> 2), p = t & 3, x = x0 + i;
             const int ti = (i & 31) + 1;
-            const uint32_t *tw = reinterpret_cast<const uint32_t *>(T + i * L::kTPitch) + (ti >> 2) +
-                                 (DP / 4 - 2 * CPP * (p + 1));
+            const uint32_t *trow32 = reinterpret_cast<const uint32_t *>(T + i * L::kTPitch) + (ti >> 2);
             const uint32_t sh = 8u * (uint32_t)(ti & 3);
-            uint32_t U[2 * CPP];
-            uint32_t prev = tw[0];
+            uint32_t lo[CPP], hi[CPP];
+            {
+                const uint32_t *tl = trow32 + DP / 4 - CPP * (p + 1), *th = trow32 + CPP * p;
+                uint32_t pl = tl[0], ph = th[0];
 #pragma unroll
-            for (int m = 0; m < 2 * CPP; m++) {
-                const uint32_t nx = tw[m + 1];
-                U[m] = __funnelshift_r(prev, nx, sh);
-                prev = nx;
+                for (int m = 0; m < CPP; m++) {
+                    const uint32_t nl = tl[m + 1], nh = th[m + 1];
+                    lo[CPP - 1 - m] = __funnelshift_r(pl, nl, sh);
+                    hi[m] = __funnelshift_r(ph, nh, sh);
+                    pl = nl;
+                    ph = nh;
+                }
             }
             const bool edge = RAGGED || x < DP - 1;
             uint32_t c[2 * CPP];
 #pragma unroll
             for (int m = 0; m < CPP; m++) {
-                const int q = CPP * p + m;
-                const uint32_t hi = U[2 * CPP - 2 - 2 * m], lo = U[2 * CPP - 1 - 2 * m];
-                uint32_t c0 = __byte_perm(hi, lo, 0x2367), c1 = __byte_perm(hi, lo, 0x0145);
+                const int j = CPP * p + m;
                 if (edge) {
 #pragma unroll
-                    for (int e = 0; e < 8; e++) {
-                        const int d = 8 * q + e;
-                        if ((RAGGED && d >= D) || x - d < 0) {
-                            const int pos = chunk_byte(8, e);
-                            const uint32_t mk = 0xFFu << (8 * (pos & 3));
-                            if (pos < 4) c0 = (c0 & ~mk) | ((uint32_t)nbits << (8 * (pos & 3)));
-                            else c1 = (c1 & ~mk) | ((uint32_t)nbits << (8 * (pos & 3)));
-                        }
+                    for (int e = 0; e < 4; e++) {
+                        const int dl = 4 * j + e, dh = DP - 1 - dl;
+                        const uint32_t ml = 0xFFu << (8 * (3 - e)), mh = 0xFFu << (8 * e);
+                        if (RAGGED && dl >= D) lo[m] = (lo[m] & ~ml) | (kPadCost << (8 * (3 - e)));
+                        else if (x - dl < 0) lo[m] = (lo[m] & ~ml) | ((uint32_t)nbits << (8 * (3 - e)));
+                        if (RAGGED && dh >= D) hi[m] = (hi[m] & ~mh) | (kPadCost << (8 * e));
+                        else if (x - dh < 0) hi[m] = (hi[m] & ~mh) | ((uint32_t)nbits << (8 * e));
                     }
                 }
-                c[2 * m] = c0;
-                c[2 * m + 1] = c1;
+                c[2 * m] = __byte_perm(lo[m], hi[m], 0x4532);
+                c[2 * m + 1] = __byte_perm(lo[m], hi[m], 0x6710);
             }
             unsigned char *rec = O + i * DP + p * (8 * CPP);
             if constexpr (CPP == 1) {
@@ -469,7 +468,7 @@ cudaError_t launch_kb(const void *codes, int W, int H, int D, int nbits, uint8_t
 
 bool cost_mma_supported(int D) {
     const int Dp = padded_disparities(D);
-    return disparities_per_lane(D) == 8 && (Dp == 32 || Dp == 64 || Dp == 128);
+    return Dp == 32 || Dp == 64 || Dp == 128;
 }
 
 cudaError_t launch_cost_mma(const void *codes, int code_bytes, int W, int H, int D, int nbits, uint8_t *cost,

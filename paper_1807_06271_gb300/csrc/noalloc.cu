@@ -146,8 +146,8 @@ extern "C" int sgm_compute_static(int W, int H, int D, const sgm_params *params,
     uint8_t *planes = base + at.planes;
     unsigned *counter = reinterpret_cast<unsigned *>(base + at.job_state);
     uint8_t *disp_lr = base + at.disp_lr;
-    const int cpl = sgm::chunks_per_lane_max(D, wide);
-    const sgm::PathJobs jobs = sgm::make_path_jobs(W, H, D, params->path_mask, cpl);
+    const int cpl = 1;
+    const sgm::PathJobs jobs = sgm::make_path_jobs(W, H, D, params->path_mask, wide, cpl);
 
     // Every kernel below overwrites the scratch it later reads, and the cost
     // kernel clears the aggregation's work-queue state, so nothing left by an

@@ -1,8 +1,9 @@
 // SAD matching cost (Sec. 3.1.2: the pixel-wise sum of absolute differences,
 // over the 5 x 5 support region of Sec. 4.1):
 //     C(x,y,d) = sum over |u| <= rw, |v| <= rh of |I_l(x+u, y+v) - I_r(x-d+u, y+v)|
-// with both images read at clamped (replicated) coordinates, and the maximum
-// cmax = ww * wh * 255 where x - d < 0 and in the padding slots d >= D.
+// with both images read at clamped (replicated) coordinates, the maximum
+// cmax = ww * wh * 255 where x - d < 0, and kPadCostWide in the padding slots
+// d >= D.
 //
 // One CTA per segment of kSeg pixels of kRows consecutive rows.  The left
 // rows (kSeg + 2 rw columns) and right rows (kSeg + Dp - 1 + 2 rw columns)
@@ -18,9 +19,10 @@
 // that leaves).  |a - b| = max.u16x2 - min.u16x2 (full rate on GB300).
 // Each row's costs then add ww neighbouring columns of V, four packed adds
 // per chunk and column (halves never carry: a cost is at most
-// ww * wh * 255 <= 32766), and go out as one 16-byte chunk per (pixel, lane)
-// in the wide lane-chunk order; consecutive threads write consecutive chunks
-// of the segment's contiguous pixel records.
+// ww * wh * 255 <= 32766).  The chunks go through a shared tile, from which
+// each 16-byte quarter of a folded record takes the halves of two chunks
+// from either end of the disparity range; consecutive threads write
+// consecutive quarters of the segment's contiguous pixel records.
 #include "sgm_internal.cuh"
 
 namespace sgm {
@@ -69,8 +71,7 @@ __global__ void __launch_bounds__(kThreads)
                     uint4 *__restrict__ cost, unsigned *__restrict__ job_state) {
     extern __shared__ __align__(16) unsigned char sad_smem[];
     wait_for_predecessor();
-    if (job_state && blockIdx.x == 0 && blockIdx.y == 0)
-        for (int i = threadIdx.x; i < (int)(kJobStateBytes / sizeof(unsigned)); i += kThreads) job_state[i] = 0u;
+    if (job_state && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *job_state = 0u;
     const int rw = ww / 2, rh = wh / 2;
     const int ncol = kSeg + 2 * rw;          // V columns (segment + halo)
     const int lcols = ncol, rcols = kSeg + Dp - 1 + 2 * rw;
@@ -79,7 +80,8 @@ __global__ void __launch_bounds__(kThreads)
     const int nrows = min(kRows, H - y0);   // output rows of this CTA
     const int srows = nrows + wh - 1;       // staged rows: y0 - rh .. y0 + nrows - 1 + rh
     uint4 *V = reinterpret_cast<uint4 *>(sad_smem);                              // [ncol][chunks]
-    uint32_t *Lp = reinterpret_cast<uint32_t *>(V + (size_t)ncol * chunks);      // [srows][lcols]: (l, l)
+    uint4 *tile = V + (size_t)ncol * chunks;                                      // [kSeg][chunks] costs of a row
+    uint32_t *Lp = reinterpret_cast<uint32_t *>(tile + (size_t)kSeg * chunks);   // [srows][lcols]: (l, l)
     uint8_t *Rb = reinterpret_cast<uint8_t *>(Lp + srows * lcols);               // [srows][rcols] bytes
     uint32_t *Rp = reinterpret_cast<uint32_t *>(Rb + ((srows * rcols + 3) & ~3));  // [srows][rcols]: (R[c], R[c-4])
     const int xl0 = x0 - rw;            // image column of left column 0
@@ -124,8 +126,7 @@ __global__ void __launch_bounds__(kThreads)
             V[it] = v;
         }
         __syncthreads();
-        // C(x, d) = sum over u < ww of V(x - x0 + u, d); cmax where x - d < 0 or d >= D.
-        uint4 *out = cost + ((size_t)(y0 + r) * W + x0) * chunks;
+        // C(x, d) = sum over u < ww of V(x - x0 + u, d); cmax where x - d < 0.
         for (int it = threadIdx.x; it < npx * chunks; it += kThreads) {
             const int px = it / chunks, i = it - px * chunks;
             uint32_t s[4] = {0u, 0u, 0u, 0u};
@@ -141,13 +142,24 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
                     const int dlo = 8 * i + k, dhi = dlo + 4;
-                    const bool mlo = dlo >= D || x - dlo < 0, mhi = dhi >= D || x - dhi < 0;
-                    s[k] = (mlo ? cmax : (s[k] & 0xFFFFu)) | ((mhi ? cmax : (s[k] >> 16)) << 16);
+                    const uint32_t vlo = dlo >= D ? kPadCostWide : x - dlo < 0 ? cmax : (s[k] & 0xFFFFu);
+                    const uint32_t vhi = dhi >= D ? kPadCostWide : x - dhi < 0 ? cmax : (s[k] >> 16);
+                    s[k] = vlo | (vhi << 16);
                 }
             }
-            out[it] = make_uint4(s[0], s[1], s[2], s[3]);
+            tile[it] = make_uint4(s[0], s[1], s[2], s[3]);
         }
         __syncthreads();
+        // Quarter q of a record: pairs 4q + e = disparities (4q + e, Dp-1-4q-e), e < 4:
+        // half q % 2 of the chunk q / 2, and the other half of its mirror image backwards.
+        uint4 *out = cost + ((size_t)(y0 + r) * W + x0) * chunks;
+        for (int it = threadIdx.x; it < npx * chunks; it += kThreads) {
+            const int px = it / chunks, q = it - px * chunks;
+            const uint4 l = tile[px * chunks + (q >> 1)], h = tile[px * chunks + chunks - 1 - (q >> 1)];
+            const uint32_t sel = q & 1 ? 0x5432u : 0x7610u;
+            out[it] = make_uint4(__byte_perm(l.x, h.w, sel), __byte_perm(l.y, h.z, sel), __byte_perm(l.z, h.y, sel),
+                                 __byte_perm(l.w, h.x, sel));
+        }
     }
 }
 
@@ -156,13 +168,13 @@ __global__ void __launch_bounds__(kThreads)
 cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch, int W, int H,
                             int D, int ww, int wh, const RectMaps &maps, uint16_t *cost,
                             unsigned *job_state, cudaStream_t s) {
-    if (disparities_per_lane(D) != 8 || ww < 1 || wh < 1 || ww > kMaxSadWindow || wh > kMaxSadWindow)
+    if (ww < 1 || wh < 1 || ww > kMaxSadWindow || wh > kMaxSadWindow)
         return cudaErrorInvalidValue;
     const int Dp = padded_disparities(D);
     const int rw = ww / 2;
     const int ncol = kSeg + 2 * rw, rcols = kSeg + Dp - 1 + 2 * rw;
     const size_t srows = (size_t)kRows + wh - 1;
-    const size_t smem = (size_t)ncol * (Dp / 8) * sizeof(uint4) + srows * ncol * 4 +
+    const size_t smem = (size_t)(ncol + kSeg) * (Dp / 8) * sizeof(uint4) + srows * ncol * 4 +
                         ((srows * rcols + 3) & ~(size_t)3) + srows * rcols * 4;
     const dim3 grid((W + kSeg - 1) / kSeg, (H + kRows - 1) / kRows);
     uint4 *out = reinterpret_cast<uint4 *>(cost);

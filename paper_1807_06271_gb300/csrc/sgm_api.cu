@@ -143,8 +143,7 @@ int run_matching(sgm_handle_s *h, const uint8_t *left, const uint8_t *right, cud
 // All enabled directions into h->planes, or direction only_r alone into plane 0.
 int run_aggregate(sgm_handle_s *h, int only_r, cudaStream_t s) {
     const int mask = only_r >= 0 ? (1 << only_r) : h->p.path_mask;
-    const PathJobs jobs = h->agg_cpl == kMixedCpl ? make_path_jobs_mixed(h->W, h->H, h->D, mask, 1, 2)
-                                                  : make_path_jobs(h->W, h->H, h->D, mask, h->agg_cpl);
+    const PathJobs jobs = make_path_jobs(h->W, h->H, h->D, mask, h->wide != 0, h->agg_cpl);
     TimingRecord *t = stage_begin(h, kStageAggregate, s);
     cudaError_t e = launch_aggregate(h->cost, h->W, h->H, h->D, h->p.P1, h->p.P2, h->wide != 0, jobs, h->planes,
                                      only_r >= 0 ? 1 : h->npaths, h->job_counter, h->agg_blocks_per_sm, h->agg_cpl, s);
@@ -342,8 +341,10 @@ int sgm_create(int W, int H, int D, const sgm_params *params, sgm_handle *out) {
     for (int r = 0; r < kMaxPaths; r++)
         if ((params->path_mask >> r) & 1) h->path_of_plane[h->npaths++] = r;
     h->Dp = padded_disparities(D);
-    h->agg_blocks_per_sm = 3;  // 12 resident warps per SM (fastest on 1242 x 375, D = 128)
-    h->agg_cpl = 1;  // one 8-disparity chunk per lane: fastest for single pairs on every measured shape
+    // 16 resident warps per SM (1242 x 375, D = 128, 8 paths: 128 us, against 133 with
+    // 12, 145 with 8 and 127 with 20); small images fill fewer
+    h->agg_blocks_per_sm = 4;
+    h->agg_cpl = 1;  // fastest for single pairs on every measured shape but portraits
     h->schedule = SGM_SCHEDULE_PLANES;
     h->sweep_rows = 4;
     const Tuning tuned = tuned_for(h);

@@ -55,7 +55,7 @@ struct sgm_handle_s {
 
     // scratch, owned
     void *codes;        // [2][H][W] census codes (left, right); null for SAD
-    uint8_t *cost;      // [H][W][Dp] matching cost, lane-chunk order (bytes, or uint16 when wide)
+    uint8_t *cost;      // [H][W][Dp] matching cost, folded records (bytes, or uint16 when wide)
     uint8_t *planes;    // [H][W][npaths][Dp] per-path aggregated costs, same order
     uint8_t *disp_lr;   // [H][W] after the LR check, before the median
     unsigned *job_counter;  // work-queue state of the aggregation kernel (kJobStateBytes), then dev_status

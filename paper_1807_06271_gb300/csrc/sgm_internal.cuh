@@ -110,59 +110,63 @@ __device__ __forceinline__ uint8_t rect_pixel(const uint8_t *__restrict__ img, i
     }
 }
 
-// Disparity layout.  The D disparities of a pixel are held by LPS lanes
-// ("lanes per scanline", a power of two) with DPL = 8 disparities each, so a
-// pixel owns Dp = DPL * LPS slots in the cost volume and in every path plane;
-// slots d >= D are padding.  A lane's chunk (disparities DPL*i .. DPL*i + DPL-1)
-// is stored so that the aggregation kernel gets the packed 16-bit pairs
-// (d+k, d+k+h), h = DPL/2, it works on with at most one mask or byte-permute:
-//   8-bit costs (census): DPL/4 32-bit words, word w holding the bytes
-//     d+2w  d+2w+1  d+2w+h  d+2w+1+h  (mask 0x00FF00FF, or permute, per pair);
-//   16-bit costs (SAD, "wide"): DPL/2 32-bit words, word k holding the
-//     uint16 pair (d+k, d+k+h) itself.
-// The kernels are written for any DPL that is a multiple of 4; 16 per lane was
-// measured slower on the 1242 x 375, D = 128 workload (fewer, fatter warps
-// lengthen the horizontal scanlines, which set the aggregation's duration), so
-// 8 is used for every D.
-inline int disparities_per_lane(int) { return 8; }
-inline int lanes_per_scanline(int D) {
-    const int dpl = disparities_per_lane(D);
-    int need = (D + dpl - 1) / dpl, l = 1;
+// Disparity layout.  A pixel owns Dp slots in the cost volume and in every path
+// plane (8 times a power of two, at least D); slots d >= D are padding.  The
+// record is folded: pair k (0 <= k < Dp/2) holds the disparities (k, Dp-1-k), so
+// that a pair's neighbours in both halves are the pairs k-1 and k+1, whatever
+// number of consecutive pairs a lane of the aggregation kernel holds.
+//   8-bit costs (census): 32-bit word w holds pairs 2w and 2w+1 as the bytes
+//     2w+1  2w  Dp-2-2w  Dp-1-2w  (the upper halves in increasing order);
+//   16-bit costs (SAD, "wide"): word k holds pair k, the lower half first.
+inline int lanes_per_scanline(int D) {  // 8-disparity chunks of a pixel
+    int need = (D + 7) / 8, l = 1;
     while (l < need) l *= 2;
     return l;
 }
-inline int padded_disparities(int D) { return disparities_per_lane(D) * lanes_per_scanline(D); }
-__host__ __device__ constexpr int chunk_byte(int dpl, int j) {  // byte of disparity dpl*i + j
-    return j < dpl / 2 ? 4 * (j / 2) + (j % 2) : 4 * ((j - dpl / 2) / 2) + 2 + ((j - dpl / 2) % 2);
+inline int padded_disparities(int D) { return 8 * lanes_per_scanline(D); }
+// Slot (byte, or uint16 for wide) of disparity d in a pixel's record.
+__host__ __device__ constexpr int fold_slot(int d, int Dp, bool wide) {
+    const int hi = d >= Dp / 2, k = hi ? Dp - 1 - d : d;
+    return wide ? 2 * k + hi : 4 * (k / 2) + 1 - k % 2 + 2 * hi;
 }
+// Cost of the padding slots.  With it they never hold a scanline's minimum nor
+// help a neighbour (census bits + P2 <= 255; SAD cmax + P2 < 0x7FFF).
+constexpr unsigned kPadCost = 255u, kPadCostWide = 0x7FFFu;
+// Planes one after the other, or all planes of a pixel back to back.
+constexpr bool kPlanar = false;
 
-// Work list of the aggregation kernel: entry k is one enabled direction whose
-// nlines scanlines are cut into jobs of G = 32 / LPS neighbouring scanlines
-// (one warp each).  Job j belongs to entry k when jbegin[k] <= j < jbegin[k+1].
+// Pairs of disparities a lane of the aggregation kernel holds, for the
+// long-axis scanlines and for the other directions, under the
+// sgm_set_aggregation setting cpl.
+struct LaneConfig {
+    int np_long, np_other;
+};
+LaneConfig lane_config(int D, bool wide, int cpl);
+inline int lanes_of(int D, int np) { return padded_disparities(D) / (2 * np); }
+
+// Work list of the aggregation kernel: entry k is one enabled direction, or a
+// direction and its opposite, whose nlines scanlines are cut into jobs of G
+// neighbouring scanlines (one warp each, G = 32 / lanes per scanline); the jobs
+// of the two directions alternate.  Job j belongs to entry k when jbegin[k] <=
+// j < jbegin[k+1].
 struct PathJobs {
-    int n;                     // number of entries
-    int dx[kMaxPaths], dy[kMaxPaths];
-    int plane[kMaxPaths];      // output plane of entry k
-    int nlines[kMaxPaths];
-    int cpl[kMaxPaths];        // 8-disparity chunks per lane of entry k's jobs
-    int jbegin[kMaxPaths + 1];
-    int nlong;                 // jobs [0, nlong) belong to the long-axis directions
-    uint32_t unit;             // always 1; see the kernel's multiply-adds
+    int n;                       // number of entries
+    int ndir[kMaxPaths / 2];     // directions of entry k
+    int dx[kMaxPaths / 2][2], dy[kMaxPaths / 2][2];
+    int plane[kMaxPaths / 2][2];  // their output planes
+    int nlines[kMaxPaths / 2];
+    int jbegin[kMaxPaths / 2 + 1];
+    int nlong;                   // jobs [0, nlong) belong to the long-axis directions
+    uint32_t unit;               // always 1; see the kernel's multiply-adds
 };
 
-// Work-queue state of the aggregation kernel (cleared before every launch):
-// word 0 hands out the long-axis jobs, word 1 the others, and words
-// kJobClaimBase + slot are claim flags, one per (SM, warp scheduler).
-constexpr int kJobClaimBase = 32, kJobClaimSlots = 1024;
-constexpr size_t kJobStateBytes = (size_t)(kJobClaimBase + kJobClaimSlots) * sizeof(unsigned);
+// Work-queue state of the aggregation kernel: word 0 counts the jobs handed out
+// beyond the warps' first ones (cleared before every launch).
+constexpr size_t kJobStateBytes = 4224;
 
 // Builds the work list for the directions in `mask` (planes numbered in
-// increasing direction order), longest scanlines first, for lanes holding
-// `cpl` 8-disparity chunks each: G = 32 / (lanes_per_scanline(D) / cpl).
-PathJobs make_path_jobs(int W, int H, int D, int mask, int cpl);
-// The same with the long-axis directions (rows when W >= H) at cpl_long chunks
-// per lane and the others at cpl_other.
-PathJobs make_path_jobs_mixed(int W, int H, int D, int mask, int cpl_long, int cpl_other);
+// increasing direction order), longest scanlines first.
+PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl);
 // The most chunks per lane the aggregation takes for D (1 for 16-bit costs, up to 4).
 int chunks_per_lane_max(int D, bool wide);
 // Chunks-per-lane code of the mixed layout: long-axis scanlines at 1, the others at 2.
@@ -172,9 +176,7 @@ constexpr int kMixedCpl = SGM_AGG_CHUNKS_MIXED;
 struct BatchAggPair {
     const void *cost;  // the pair's cost volume
     void *planes;      // its path planes
-    int W, H, D;
-    int lps;           // lanes per scanline: the pixel's chunks / chunks per lane
-    int ragged;        // D < 8 * lps
+    int W, H, Dp;
     int nplanes;
     PathJobs jobs;
 };
@@ -187,7 +189,7 @@ namespace sgm {
 cudaError_t launch_census(const uint8_t *left, const uint8_t *right, int pitch, int W, int H,
                           int cw, int ch, int code_bytes, void *codes, const RectMaps &maps,
                           cudaStream_t s);
-// The cost kernels also clear job_state (kJobStateBytes, may be null), the
+// The cost kernels also clear word 0 of job_state (may be null), the
 // work-queue state of the aggregation kernel that follows them on the stream.
 // Hamming costs of the census codes come from one of two kernels (kernel:
 // SGM_COST_KERNEL_*): POPC on the CUDA cores (any D) or +-1 inner products on
@@ -203,7 +205,7 @@ cudaError_t launch_cost_mma(const void *codes, int code_bytes, int W, int H, int
 // The kernel SGM_COST_KERNEL_AUTO selects for D.
 int cost_kernel_for(int D);
 // SAD over a ww x wh window (clamped reads; rectified through maps when set) into a
-// 16-bit cost volume [H][W][Dp] in the wide lane-chunk order.
+// 16-bit cost volume [H][W][Dp] of folded records.
 cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch, int W, int H,
                             int D, int ww, int wh, const RectMaps &maps, uint16_t *cost,
                             unsigned *job_state, cudaStream_t s);
@@ -222,7 +224,7 @@ cudaError_t launch_aggregate(const uint8_t *cost, int W, int H, int D, int P1, i
 // cpl: 1 or 4 (4 only for 8-bit costs and pairs whose D allows it).
 cudaError_t launch_aggregate_batch(const BatchAggPair *pairs, int npairs, const int *prefix, int P1, int P2,
                                    bool wide, int cpl, unsigned *job_counter, int blocks_per_sm, cudaStream_t s);
-// Copies a single plane ([H][W][Dp], lane-chunk order) to L ([H][W][D] uint16, natural order).
+// Copies a single plane ([H][W][Dp], folded records) to L ([H][W][D] uint16, natural order).
 cudaError_t launch_unpermute(const uint8_t *plane, int W, int H, int D, bool wide, uint16_t *L,
                              cudaStream_t s);
 cudaError_t launch_wta(const uint8_t *planes, int nplanes, int W, int H, int D, bool wide,

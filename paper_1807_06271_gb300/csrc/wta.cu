@@ -2,12 +2,12 @@
 // disparity taken from the same S (Sec. 3.1.4) and the left-right check.
 //
 // One CTA per image row.  The planes share the aggregation kernel's layout
-// (all planes of a pixel back to back): LPS lanes hold a pixel's
-// disparities, DPL per lane, so a warp covers G = 32 / LPS neighbouring
+// (all planes of a pixel back to back, folded records): LPS lanes hold a
+// pixel's disparities, DPL per lane, so a warp covers G = 32 / LPS neighbouring
 // pixels.  A lane loads its chunk of every plane (8 bytes of 8-bit path
 // costs, or 16 bytes of 16-bit ones) at fixed offsets from one pointer, one
 // or two pixel groups ahead of its use (register buffers), turns each into
-// DPL/2 packed 16-bit pairs (d+k, d+k+DPL/2) (masks and byte-permutes for
+// DPL/2 packed 16-bit pairs (d, Dp-1-d) (masks and byte-permutes for
 // 8-bit planes; 16-bit planes are stored that way) and adds them.  No half
 // carries: S <= 8 * 255 for 8-bit planes, and the host bounds the 16-bit
 // path costs so that their sum fits 16 bits.  For each disparity it forms the
@@ -76,26 +76,26 @@ __device__ __forceinline__ PlaneChunk<DPL, WIDE> ld_plane(const uint8_t *p, uint
     return v;
 }
 
-// XOR mask on the lane's visiting order of its disparities: with it the
-// shared-memory atomics that a warp issues together fall into distinct banks
-// (checked exhaustively for every (DPL, LPS) in use).
-template <int DPL, int LPS>
+// XOR mask on the lane's visiting order of its pairs.  The slots that the lanes
+// of a pixel address together are four apart, so lanes eight apart share a bank;
+// with the mask they (and the two pixels of a 16-lane warp) fall into distinct
+// banks.
+template <int LPS>
 __device__ __forceinline__ int visit_mask(int li) {
-    static_assert(DPL == 8, "masks are tabulated for 8 disparities per lane");
-    if constexpr (LPS == 8) return 4 * ((li >> 2) & 1);
-    else if constexpr (LPS == 16) return 2 * ((li >> 2) & 3);
-    else if constexpr (LPS == 32) return ((li >> 2) & 3) + 4 * ((li >> 4) & 1);
+    if constexpr (LPS == 16) return 2 * ((li >> 3) & 1);
+    else if constexpr (LPS == 32) return (li >> 3) & 3;
     else return 0;
 }
 
-// Sums the path planes of one pixel into DPL/2 packed pairs S[k] = (S(d0+k), S(d0+k+h)),
-// h = DPL/2, folds its keys into the right-disparity slots and returns its smallest key.
+// Sums the path planes of one pixel into DPL/2 packed pairs
+// S[k] = (S(d), S(Dp-1-d)), d = li * DPL/2 + k, folds its keys into the
+// right-disparity slots and returns its smallest key.
 // NP > 0: NP planes (compile time); NP == 0: nplanes at run time.
 template <int LPS, int DPL, bool WIDE, int NP, bool RAGGED, bool DEBUG>
 __device__ __forceinline__ uint32_t pixel_keys(const PlaneChunk<DPL, WIDE> (&v)[kMaxPaths], int nplanes,
                                                bool active, int x, int y, int W, int D, int li,
                                                uint32_t *key_right, uint16_t *dbg_sum) {
-    constexpr int NR = DPL / 2;
+    constexpr int NR = DPL / 2, Dp = DPL * LPS;
     uint32_t S[NR];
 #pragma unroll
     for (int k = 0; k < NR; k++) S[k] = 0u;
@@ -104,18 +104,18 @@ __device__ __forceinline__ uint32_t pixel_keys(const PlaneChunk<DPL, WIDE> (&v)[
         if (NP > 0 || q < nplanes) {
             if constexpr (WIDE) {
 #pragma unroll
-                for (int k = 0; k < NR; k++) S[k] += v[q].w[k];  // stored as (d+k, d+k+h)
+                for (int k = 0; k < NR; k++) S[k] += v[q].w[k];
             } else {
 #pragma unroll
                 for (int w = 0; w < DPL / 4; w++) {
-                    S[2 * w] += v[q].w[w] & kLo;
-                    S[2 * w + 1] += __byte_perm(v[q].w[w], 0u, 0x4341);
+                    S[2 * w] += __byte_perm(v[q].w[w], 0u, 0x4341);
+                    S[2 * w + 1] += v[q].w[w] & kLo;
                 }
             }
         }
-    const int d0 = DPL * li;
-    const int m = visit_mask<DPL, LPS>(li);
-    // T[k] = S[k ^ (m mod NR)], halves swapped when m has the bit NR
+    const int d0 = NR * li;
+    const int m = visit_mask<LPS>(li);
+    // T[k] = S[k ^ m]
 #pragma unroll
     for (int b = 1; b < NR; b <<= 1) {
         if (m & b) {
@@ -128,16 +128,13 @@ __device__ __forceinline__ uint32_t pixel_keys(const PlaneChunk<DPL, WIDE> (&v)[
                 }
         }
     }
-    if (m & NR) {
-#pragma unroll
-        for (int k = 0; k < NR; k++) S[k] = __byte_perm(S[k], S[k], 0x1032);
-    }
     uint32_t best = 0xFFFFFFFFu;
-    // every slot x - d of this lane lies in the row when x >= d0 + DPL - 1
-    const bool inside = active && x >= d0 + DPL - 1;
+    // every slot x - d of this lane lies in the row when x >= Dp - 1 - d0
+    const bool inside = active && x >= Dp - 1 - d0;
 #pragma unroll
     for (int j = 0; j < DPL; j++) {
-        const int d = d0 + (j ^ m);
+        const int k = d0 + ((j % NR) ^ m);
+        const int d = j < NR ? k : Dp - 1 - k;
         const uint32_t sv = (j < NR) ? (S[j % NR] & 0xFFFFu) : (S[j % NR] >> 16);
         uint32_t key = sv * 256u + (uint32_t)d;
         if (RAGGED && d >= D) key = 0xFFFFFFFFu;
@@ -177,13 +174,14 @@ __global__ void __launch_bounds__(kThreads, PF == 2 ? 2 : 1)
     __syncthreads();
     // pixel records hold all planes of a pixel back to back: nplanes * Dp * EB bytes
     const int np = NP > 0 ? NP : nplanes;
-    const size_t rec = (size_t)np * Dp * EB;
+    const size_t rec = (kPlanar ? (size_t)1 : (size_t)np) * Dp * EB;
+    const size_t pstep = kPlanar ? (size_t)W * H * Dp * EB : (size_t)Dp * EB;
     const uint8_t *row = planes + (size_t)y * W * rec + DPL * EB * li;
     const uint64_t pol = policy_evict_first();
     const int stride = nwarps * G;
     // byte offset of a lane's chunk from `planes`, and the last one that fits
     const long long row_off = (long long)y * W * (long long)rec + DPL * EB * li;
-    const long long chunk_limit = (long long)W * H * (long long)rec - DPL * EB + 1;
+    const long long chunk_limit = (long long)W * H * np * Dp * EB - DPL * EB + 1;
     // software pipeline: the planes of the next PF pixel groups are loaded
     // while the current one is reduced (buf[0] is the current group)
     static_assert(PF == 1 || PF == 2, "one or two pixel groups ahead");
@@ -200,14 +198,14 @@ __global__ void __launch_bounds__(kThreads, PF == 2 ? 2 : 1)
 #pragma unroll
         for (int q = 0; q < NQ; q++)
             if ((NP > 0 || q < np) && x + b * stride < W &&
-                in_range(row_off + (long long)(x + b * stride) * (long long)rec + q * Dp * EB, chunk_limit))
-                buf[b][q] = ld_plane<DPL, WIDE>(row + (size_t)(x + b * stride) * rec + q * Dp * EB, pol);
+                in_range(row_off + (long long)(x + b * stride) * (long long)rec + (long long)(q * pstep), chunk_limit))
+                buf[b][q] = ld_plane<DPL, WIDE>(row + (size_t)(x + b * stride) * rec + q * pstep, pol);
     for (int xb = warp * G; xb < W; xb += stride) {
         const int xn = x + stride, xf = x + PF * stride;
 #pragma unroll
         for (int q = 0; q < NQ; q++)
-            if ((NP > 0 || q < np) && xf < W && in_range(row_off + (long long)xf * (long long)rec + q * Dp * EB, chunk_limit))
-                buf[PF][q] = ld_plane<DPL, WIDE>(row + (size_t)xf * rec + q * Dp * EB, pol);
+            if ((NP > 0 || q < np) && xf < W && in_range(row_off + (long long)xf * (long long)rec + (long long)(q * pstep), chunk_limit))
+                buf[PF][q] = ld_plane<DPL, WIDE>(row + (size_t)xf * rec + q * pstep, pol);
         const bool active = x < W;
         uint32_t best = pixel_keys<LPS, DPL, WIDE, NP, RAGGED, DEBUG>(buf[0], np, active, x, y, W, D, li, key_right, dbg_sum);
         best = group_min<LPS>(best, lane);
@@ -306,7 +304,6 @@ SGM_GUARD_COUNTER(guard_hits_wta)
 cudaError_t launch_wta(const uint8_t *planes, int nplanes, int W, int H, int D, bool wide,
                        int tol, uint8_t *disp_lr, uint8_t *dbg_left, uint8_t *dbg_right,
                        uint16_t *dbg_sum, cudaStream_t s) {
-    if (disparities_per_lane(D) != 8) return cudaErrorInvalidValue;
     const size_t smem = (size_t)W * sizeof(uint32_t) + (size_t)((W + 3) & ~3);
     if (wide) return launch_wta_t<true>(planes, nplanes, W, H, D, tol, disp_lr, dbg_left, dbg_right, dbg_sum, smem, s);
     return launch_wta_t<false>(planes, nplanes, W, H, D, tol, disp_lr, dbg_left, dbg_right, dbg_sum, smem, s);
