@@ -69,9 +69,10 @@ namespace sgm {
 
 LaneConfig lane_config(int D, bool wide, int cpl) {
     const int Dp = padded_disparities(D);
-    if (!wide && cpl == 2) return {8, 8};
-    if (!wide && cpl == 4) return {16, 16};
-    if (!wide && cpl == kMixedCpl) return {4, 8};
+    const bool pow2 = (Dp & (Dp - 1)) == 0;  // lanes of more than 4 pairs come in powers of two
+    if (!wide && pow2 && cpl == 2) return {8, 8};
+    if (!wide && pow2 && cpl == 4) return {16, 16};
+    if (!wide && pow2 && cpl == kMixedCpl) return {4, 8};
     return {Dp <= 128 ? 2 : 4, 4};
 }
 
@@ -373,7 +374,8 @@ __device__ __forceinline__ void line_start(int dx, int dy, int s, int W, int H, 
 // One job: the G neighbouring scanlines s0 .. s0+G-1 of one direction
 // (dx, dy), scanline s0 + grp for this lane's group, written to plane
 // `plane` of `nplanes`.  A scanline's pixel is LPS lane blocks of NP pairs.
-template <int NP, int G, bool WIDE>
+// FULL: the G scanlines' lanes fill the warp.
+template <int NP, int G, bool WIDE, bool FULL>
 __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__restrict__ planes_, int W, int H,
                                         int lps_, int nplanes, int dx, int dy, int plane, int nlines, int s0,
                                         uint32_t P1x2, uint32_t P2x2, uint64_t pol, uint32_t one) {
@@ -381,20 +383,22 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     using RT = Ring<NP, G, WIDE>;
     extern __shared__ __align__(16) uint8_t agg_smem[];
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(agg_smem) + (threadIdx.x >> 5) * kRingBytes;
-    const int LPS = G >= 8 ? 32 / G : lps_;
+    const int LPS = G >= 8 || FULL ? 32 / G : lps_;
     const int lane = threadIdx.x & 31;
     LaneGeom lg;
-    lg.grp = lane / LPS;
-    lg.li = lane - lg.grp * LPS;
+    // Lanes beyond the last scanline repeat its last lane, in all it computes and stores.
+    const int vl = FULL ? lane : min(lane, G * LPS - 1);
+    lg.grp = vl / LPS;
+    lg.li = vl - lg.grp * LPS;
     lg.first = lg.li == 0;
     const bool last = lg.li == LPS - 1;
-    lg.src_up = lg.first ? lane : lane - 1;
-    lg.src_dn = last || lane == 31 ? lane : lane + 1;
+    lg.src_up = lg.first ? lane : vl - 1;
+    lg.src_dn = last ? lane : lane + 1;
     lg.sel_dn = last ? 0x5476u : 0x3210u;
     lg.lo_mark = lg.first ? 0x7FFF7FFFu : 0u;
     const int s = s0 + lg.grp;
     int x = 0, y = 0, len = 0;
-    if (lg.grp < G && s < nlines) line_start(dx, dy, s, W, H, x, y, len);
+    if (s < nlines) line_start(dx, dy, s, W, H, x, y, len);
     const int steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
     const int minlen = (int)__reduce_min_sync(0xffffffffu, (unsigned)len);
     // block indices: cost block (x, y, li) is cost[(y*W + x)*LPS + li], plane
@@ -411,6 +415,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     const int rec = LPS * (int)sizeof(BT);  // bytes of a pixel's record
     const int csub = lane * RT::kCopy / RT::kStep;
     int clen[RT::kParts];
+    bool mine[RT::kParts];  // a step's records may be shorter than the warp's copies
     uint32_t ci[RT::kParts];  // in units of kCopy bytes, below 2^32 like oi
 #pragma unroll
     for (int p = 0; p < RT::kParts; p++) {
@@ -418,11 +423,12 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
         const int cgrp = unit / rec;
         int cx = 0, cy = 0;
         clen[p] = 0;
-        if (cgrp < G && s0 + cgrp < nlines) line_start(dx, dy, s0 + cgrp, W, H, cx, cy, clen[p]);
+        mine[p] = FULL || cgrp < G;
+        if (mine[p] && s0 + cgrp < nlines) line_start(dx, dy, s0 + cgrp, W, H, cx, cy, clen[p]);
         ci[p] = (uint32_t)((((long long)cy * W + cx + csub * dir) * rec + (unit - cgrp * rec)) / RT::kCopy);
     }
     const uint32_t cadv = (uint32_t)(dir * RT::kPer * rec / RT::kCopy);
-    const uint32_t ring_w = ring + lane * RT::kCopy, ring_r = ring + lane * (int)sizeof(BT);
+    const uint32_t ring_w = ring + lane * RT::kCopy, ring_r = ring + vl * (int)sizeof(BT);
     using CT = typename std::conditional<RT::kCopy == 16, uint4, uint2>::type;
     const CT *__restrict__ cost = reinterpret_cast<const CT *>(cost_);
     BT *__restrict__ planes = reinterpret_cast<BT *>(planes_);
@@ -437,7 +443,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
                 if constexpr (decltype(checked)::value) {
                     const bool ok = blk * RT::kBlock + i + csub < clen[p] && in_range(ci[p], cost_copies);
                     copy_or_zero<RT::kCopy>(to, cost + (ok ? ci[p] : 0u), ok);
-                } else if (in_range(ci[p], cost_copies)) {
+                } else if (mine[p] && in_range(ci[p], cost_copies)) {
                     copy_async<RT::kCopy>(to, cost + ci[p]);
                 }
                 ci[p] += cadv;
@@ -497,7 +503,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
 
 // Jobs of the long-axis entry hold NPL pairs per lane (GL scanlines per warp),
 // the others NPO (GO).
-template <int NPL, int GL, int NPO, int GO, bool WIDE>
+template <int NPL, int GL, int NPO, int GO, bool WIDE, bool FULL>
 __global__ void __launch_bounds__(kWarps * 32, 5)
     aggregate_kernel(const void *__restrict__ cost, int W, int H, int Dp, uint32_t P1x2, uint32_t P2x2,
                      const __grid_constant__ PathJobs jobs, void *__restrict__ planes, int nplanes,
@@ -513,23 +519,23 @@ __global__ void __launch_bounds__(kWarps * 32, 5)
         const int q = job - jobs.jbegin[k];
         const int e = jobs.ndir[k] == 2 ? q & 1 : 0, line = jobs.ndir[k] == 2 ? q >> 1 : q;
         if (job < jobs.nlong)
-            run_job<NPL, GL, WIDE>(cost, planes, W, H, Dp / (2 * NPL), nplanes, jobs.dx[k][e], jobs.dy[k][e],
+            run_job<NPL, GL, WIDE, FULL>(cost, planes, W, H, Dp / (2 * NPL), nplanes, jobs.dx[k][e], jobs.dy[k][e],
                                    jobs.plane[k][e], jobs.nlines[k], line * GL, P1x2, P2x2, pol, jobs.unit);
         else
-            run_job<NPO, GO, WIDE>(cost, planes, W, H, Dp / (2 * NPO), nplanes, jobs.dx[k][e], jobs.dy[k][e],
+            run_job<NPO, GO, WIDE, FULL>(cost, planes, W, H, Dp / (2 * NPO), nplanes, jobs.dx[k][e], jobs.dy[k][e],
                                    jobs.plane[k][e], jobs.nlines[k], line * GO, P1x2, P2x2, pol, jobs.unit);
         job = next_job(job_counter, total, lane);
     }
 }
 
 // Scanlines a warp walks at once.
-constexpr int lines_per_warp(int Dp, int np) { return Dp / (2 * np) > 0 ? 32 / (Dp / (2 * np)) : 0; }
+__host__ __device__ constexpr int lines_per_warp(int Dp, int np) { return Dp / (2 * np) > 0 ? 32 / (Dp / (2 * np)) : 0; }
 
 // Many pairs in one persistent launch.  The work list of pair p is its
 // PathJobs; the two queues number all pairs' long-axis jobs (queue 0) and
 // all their other jobs (queue 1) in pair order, pair p's starting at
 // pfx[0][p] and pfx[1][p].  Each job runs with its pair's lanes per scanline;
-// CPL is the setting of lane_config.
+// CPL == 4 adds the lanes of 16 pairs.
 template <int CPL, bool WIDE>
 __global__ void __launch_bounds__(kWarps * 32, 5)
     aggregate_batch_kernel(const BatchAggPair *__restrict__ pairs, int npairs, const int *__restrict__ prefix,
@@ -563,59 +569,79 @@ __global__ void __launch_bounds__(kWarps * 32, 5)
         const int e = p.jobs.ndir[k] == 2 ? ql & 1 : 0, line = p.jobs.ndir[k] == 2 ? ql >> 1 : ql;
         auto job_as = [&](auto np, auto g) {
             constexpr int NP = decltype(np)::value, G = decltype(g)::value;
-            run_job<NP, G, WIDE>(p.cost, p.planes, p.W, p.H, p.Dp / (2 * NP), p.nplanes, p.jobs.dx[k][e],
+            run_job<NP, G, WIDE, (G >= 8)>(p.cost, p.planes, p.W, p.H, p.Dp / (2 * NP), p.nplanes, p.jobs.dx[k][e],
                                  p.jobs.dy[k][e], p.jobs.plane[k][e], p.jobs.nlines[k], line * G, P1x2, P2x2, pol,
                                  p.jobs.unit);
         };
-#define SGM_JOB(DPV)                                                                                            \
-    case DPV: {                                                                                                 \
-        constexpr int npl = CPL == 4 ? 16 : (DPV <= 128 ? 2 : 4), npo = CPL == 4 ? 16 : 4;                      \
-        if constexpr (DPV >= 2 * npl && DPV >= 2 * npo) {                                                       \
-            if (lq) job_as(std::integral_constant<int, npl>(), std::integral_constant<int, lines_per_warp(DPV, npl)>()); \
-            else job_as(std::integral_constant<int, npo>(), std::integral_constant<int, lines_per_warp(DPV, npo)>());    \
-        }                                                                                                       \
-        break;                                                                                                  \
-    }
-        switch (p.Dp) {
-            SGM_JOB(8)
-            SGM_JOB(16)
-            SGM_JOB(32)
-            SGM_JOB(64)
-            SGM_JOB(128)
-            SGM_JOB(256)
+        // pairs per lane of this job, and scanlines per warp
+        const int np = lq ? p.np_long : p.np_other;
+#define SGM_JOB(NP, G) \
+    case 64 * NP + G: job_as(std::integral_constant<int, NP>(), std::integral_constant<int, G>()); break
+        switch (64 * np + lines_per_warp(p.Dp, np)) {
+            SGM_JOB(2, 16);
+            SGM_JOB(2, 8);
+            SGM_JOB(2, 4);
+            SGM_JOB(2, 2);
+            SGM_JOB(2, 1);
+            SGM_JOB(4, 32);
+            SGM_JOB(4, 16);
+            SGM_JOB(4, 8);
+            SGM_JOB(4, 4);
+            SGM_JOB(4, 2);
+            SGM_JOB(4, 1);
+            default:
+                if constexpr (CPL == 4) switch (64 * np + lines_per_warp(p.Dp, np)) {
+                    SGM_JOB(16, 32);
+                    SGM_JOB(16, 16);
+                    SGM_JOB(16, 8);
+                    SGM_JOB(16, 4);
+                }
         }
 #undef SGM_JOB
         job = next_job(job_counter, total, lane);
     }
 }
 
-template <int NPL, int NPO, int DPV, bool WIDE>
-cudaError_t launch_dp(const void *cost, int W, int H, uint32_t P1x2, uint32_t P2x2, const PathJobs &jobs,
-                      void *planes, int nplanes, unsigned *job_counter, int blocks, int sms, cudaStream_t s) {
-    // NPL of 0: 2 pairs per lane while a warp holds the scanline, else 4
-    constexpr int npl = NPL > 0 ? NPL : DPV <= 128 ? 2 : 4;
-    if constexpr (DPV < 2 * npl || DPV < 2 * NPO) {
-        return cudaErrorInvalidValue;
-    } else {
-        return launch_k(aggregate_kernel<npl, lines_per_warp(DPV, npl), NPO, lines_per_warp(DPV, NPO), WIDE>, dim3(blocks),
-                        dim3(kWarps * 32), kWarps * kRingBytes, s, cost, W, H, DPV, P1x2, P2x2, jobs, planes, nplanes, job_counter, sms);
-    }
-}
+using AggKernel = void (*)(const void *, int, int, int, uint32_t, uint32_t, const PathJobs, void *, int, unsigned *, int);
 
-template <int NPL, int NPO, bool WIDE>
-cudaError_t launch_np(int Dp, const void *cost, int W, int H, uint32_t P1x2, uint32_t P2x2, const PathJobs &jobs,
-                      void *planes, int nplanes, unsigned *job_counter, int blocks, int sms, cudaStream_t s) {
-#define SGM_AGG(V) case V: return launch_dp<NPL, NPO, V, WIDE>(cost, W, H, P1x2, P2x2, jobs, planes, nplanes, job_counter, blocks, sms, s)
-    switch (Dp) {
-        SGM_AGG(8);
-        SGM_AGG(16);
-        SGM_AGG(32);
-        SGM_AGG(64);
-        SGM_AGG(128);
-        SGM_AGG(256);
-        default: return cudaErrorInvalidValue;
+// The kernel of a pair of lane widths, null when there is none.
+template <bool WIDE>
+AggKernel agg_kernel_t(int Dp, LaneConfig lc) {
+    const bool full = (Dp & (Dp - 1)) == 0;
+#define SGM_AGG_F(NPL, GL, NPO, GO, FULL)                                                                            \
+    if (full == FULL && lc.np_long == NPL && lc.np_other == NPO && lines_per_warp(Dp, NPL) == GL && lines_per_warp(Dp, NPO) == GO) \
+        return aggregate_kernel<NPL, GL, NPO, GO, WIDE, FULL>
+#define SGM_AGG(NPL, GL, NPO, GO) SGM_AGG_F(NPL, GL, NPO, GO, true)
+    SGM_AGG(2, 16, 4, 32);  // Dp = 8
+    SGM_AGG(2, 8, 4, 16);   // 16
+    SGM_AGG(2, 4, 4, 8);    // 32
+    SGM_AGG(2, 2, 4, 4);    // 64
+    SGM_AGG(2, 1, 4, 2);    // 128
+    SGM_AGG(4, 1, 4, 1);    // 256
+    SGM_AGG_F(2, 1, 4, 2, false);  // 96
+    SGM_AGG_F(4, 1, 4, 1, false);  // 160, 192, 224
+    if constexpr (!WIDE) {  // Dp a power of two, 16 to 256
+        SGM_AGG(8, 32, 8, 32);
+        SGM_AGG(8, 16, 8, 16);
+        SGM_AGG(8, 8, 8, 8);
+        SGM_AGG(8, 4, 8, 4);
+        SGM_AGG(8, 2, 8, 2);
+        SGM_AGG(4, 16, 8, 32);
+        SGM_AGG(4, 8, 8, 16);
+        SGM_AGG(4, 4, 8, 8);
+        SGM_AGG(4, 2, 8, 4);
+        SGM_AGG(4, 1, 8, 2);
+        SGM_AGG(16, 32, 16, 32);
+        SGM_AGG(16, 16, 16, 16);
+        SGM_AGG(16, 8, 16, 8);
+        SGM_AGG(16, 4, 16, 4);
     }
 #undef SGM_AGG
+#undef SGM_AGG_F
+    return nullptr;
+}
+AggKernel agg_kernel(int Dp, LaneConfig lc, bool wide) {
+    return wide ? agg_kernel_t<true>(Dp, lc) : agg_kernel_t<false>(Dp, lc);
 }
 
 // Plane 0 ([H][W][Dp], folded records) -> L ([H][W][D] uint16, natural order).
@@ -657,12 +683,12 @@ cudaError_t launch_aggregate(const uint8_t *cost, int W, int H, int D, int P1, i
     const int wanted = sms * (blocks_per_sm > 0 ? blocks_per_sm : 2), filled = (jobs.jbegin[jobs.n] + kWarps - 1) / kWarps;
     const int blocks = filled < sms ? sms : filled < wanted ? filled : wanted;
     const int Dp = padded_disparities(D);
+    const LaneConfig lc = lane_config(D, wide, cpl);
     const uint32_t P1x2 = (uint32_t)P1 * 0x00010001u, P2x2 = (uint32_t)P2 * 0x00010001u;
-    if (wide) return launch_np<0, 4, true>(Dp, cost, W, H, P1x2, P2x2, jobs, planes, nplanes, job_counter, blocks, sms, s);
-    if (cpl == kMixedCpl) return launch_np<4, 8, false>(Dp, cost, W, H, P1x2, P2x2, jobs, planes, nplanes, job_counter, blocks, sms, s);
-    if (cpl == 4) return launch_np<16, 16, false>(Dp, cost, W, H, P1x2, P2x2, jobs, planes, nplanes, job_counter, blocks, sms, s);
-    if (cpl == 2) return launch_np<8, 8, false>(Dp, cost, W, H, P1x2, P2x2, jobs, planes, nplanes, job_counter, blocks, sms, s);
-    return launch_np<0, 4, false>(Dp, cost, W, H, P1x2, P2x2, jobs, planes, nplanes, job_counter, blocks, sms, s);
+    auto kernel = agg_kernel(Dp, lc, wide);
+    if (!kernel) return cudaErrorInvalidValue;
+    return launch_k(kernel, dim3(blocks), dim3(kWarps * 32), kWarps * kRingBytes, s, (const void *)cost, W, H, Dp, P1x2,
+                    P2x2, jobs, (void *)planes, nplanes, job_counter, sms);
 }
 
 cudaError_t launch_aggregate_batch(const BatchAggPair *pairs, int npairs, const int *prefix, int P1, int P2,

@@ -130,6 +130,9 @@ int layout_groups(sgm_batch_s *b, int ng, bool upload, size_t at, size_t *end) {
             t.W = ps.W;
             t.H = ps.H;
             t.Dp = ps.Dp;
+            const LaneConfig lc = lane_config(ps.D, b->wide != 0, b->cpl);
+            t.np_long = lc.np_long;
+            t.np_other = lc.np_other;
             t.nplanes = b->npaths;
             t.jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl);
             prefix[k + 1] = prefix[k] + t.jobs.nlong;

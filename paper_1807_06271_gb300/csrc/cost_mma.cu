@@ -185,7 +185,7 @@ struct Smem {
 
 template <int DP, int KB, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, 1)
-    hamming_mma_kernel(const uint32_t *__restrict__ codes, int W, int H, int D, int nbits,
+    hamming_mma_kernel(const uint32_t *__restrict__ codes, int W, int H, int D, int Dp, int nbits,
                        uint8_t *__restrict__ cost, unsigned *__restrict__ job_state,
                        unsigned *__restrict__ status, int stall_test) {
     using L = Smem<DP, KB>;
@@ -359,15 +359,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         {
             // records: pixel i = 8 * warp + t / 4, word pairs CPP * p .. CPP * p + CPP - 1, p = t % 4.
             // Pixel i (lane t_i = i % 32 of its quarter) reads bytes u = 0 .. DP-1 of its T row from
-            // t_i + 1 on, u <-> d = DP - 1 - u.  Word pair j holds the disparities 4j + e and DP-1-4j-e:
-            // the four bytes from u = DP - 4 - 4j (d = 4j+3 .. 4j) and those from u = 4j (d = DP-1-4j ..).
+            // t_i + 1 on, u <-> d = DP - 1 - u.  Word pair j < Dp/8 holds the disparities 4j + e and
+            // Dp-1-4j-e: the four bytes from u = DP - 4 - 4j (d = 4j+3 .. 4j) and those from
+            // u = DP - Dp + 4j (d = Dp-1-4j ..).
             const int i = 8 * warp + (t >> 2), p = t & 3, x = x0 + i;
             const int ti = (i & 31) + 1;
             const uint32_t *trow32 = reinterpret_cast<const uint32_t *>(T + i * L::kTPitch) + (ti >> 2);
             const uint32_t sh = 8u * (uint32_t)(ti & 3);
             uint32_t lo[CPP], hi[CPP];
             {
-                const uint32_t *tl = trow32 + DP / 4 - CPP * (p + 1), *th = trow32 + CPP * p;
+                const uint32_t *tl = trow32 + DP / 4 - CPP * (p + 1), *th = trow32 + (DP - Dp) / 4 + CPP * p;
                 uint32_t pl = tl[0], ph = th[0];
 #pragma unroll
                 for (int m = 0; m < CPP; m++) {
@@ -386,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (edge) {
 #pragma unroll
                     for (int e = 0; e < 4; e++) {
-                        const int dl = 4 * j + e, dh = DP - 1 - dl;
+                        const int dl = 4 * j + e, dh = Dp - 1 - dl;
                         const uint32_t ml = 0xFFu << (8 * (3 - e)), mh = 0xFFu << (8 * e);
                         if (RAGGED && dl >= D) lo[m] = (lo[m] & ~ml) | (kPadCost << (8 * (3 - e)));
                         else if (x - dl < 0) lo[m] = (lo[m] & ~ml) | ((uint32_t)nbits << (8 * (3 - e)));
@@ -397,17 +398,18 @@ __global__ void __launch_bounds__(kThreads, 1)
                 c[2 * m] = __byte_perm(lo[m], hi[m], 0x4532);
                 c[2 * m + 1] = __byte_perm(lo[m], hi[m], 0x6710);
             }
-            unsigned char *rec = O + i * DP + p * (8 * CPP);
+            unsigned char *rec = O + i * Dp + p * (8 * CPP);
+            const int left = Dp - p * (8 * CPP);  // bytes of the record from here (a multiple of 16 where CPP > 1)
             if constexpr (CPP == 1) {
                 *reinterpret_cast<uint2 *>(rec) = make_uint2(c[0], c[1]);
             } else if constexpr (CPP == 2) {
-                *reinterpret_cast<uint4 *>(rec) = make_uint4(c[0], c[1], c[2], c[3]);
+                if (left > 0) *reinterpret_cast<uint4 *>(rec) = make_uint4(c[0], c[1], c[2], c[3]);
             } else {
                 // two 16-byte halves; the odd pixel of a pair stores them in the other order (distinct banks)
                 const bool sw = i & 1;
                 const uint4 lo4 = make_uint4(c[0], c[1], c[2], c[3]), hi4 = make_uint4(c[4], c[5], c[6], c[7]);
-                *reinterpret_cast<uint4 *>(rec + (sw ? 16 : 0)) = sw ? hi4 : lo4;
-                *reinterpret_cast<uint4 *>(rec + (sw ? 0 : 16)) = sw ? lo4 : hi4;
+                if (left > (sw ? 16 : 0)) *reinterpret_cast<uint4 *>(rec + (sw ? 16 : 0)) = sw ? hi4 : lo4;
+                if (left > (sw ? 0 : 16)) *reinterpret_cast<uint4 *>(rec + (sw ? 0 : 16)) = sw ? lo4 : hi4;
             }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -415,8 +417,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (tid == 0) {
             const int npx = min(kM, W - x0);
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
-                             cost + ((size_t)y * W + x0) * DP),
-                         "r"(smem_addr(O)), "r"(npx * DP)
+                             cost + ((size_t)y * W + x0) * Dp),
+                         "r"(smem_addr(O)), "r"(npx * Dp)
                          : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
@@ -443,8 +445,8 @@ cudaError_t launch_dp(const void *codes, int W, int H, int D, int nbits, uint8_t
     if (e != cudaSuccess) return e;
     const long long nseg = (long long)((W + kM - 1) / kM) * H;
     const int grid = nseg < sms ? (int)nseg : sms;
-    return launch_k(kernel, dim3(grid), dim3(kThreads), (size_t)smem, s, (const uint32_t *)codes, W, H, D, nbits,
-                    cost, job_state, status, stall_test);
+    return launch_k(kernel, dim3(grid), dim3(kThreads), (size_t)smem, s, (const uint32_t *)codes, W, H, D,
+                    padded_disparities(D), nbits, cost, job_state, status, stall_test);
 }
 
 template <int KB>
@@ -455,12 +457,9 @@ cudaError_t launch_kb(const void *codes, int W, int H, int D, int nbits, uint8_t
 #define SGM_MMA(P)                                                                                 \
     return rag ? launch_dp<P, KB, true>(codes, W, H, D, nbits, cost, job_state, status, stall_test, s) \
                : launch_dp<P, KB, false>(codes, W, H, D, nbits, cost, job_state, status, stall_test, s)
-    switch (Dp) {
-        case 32: SGM_MMA(32);
-        case 64: SGM_MMA(64);
-        case 128: SGM_MMA(128);
-        default: return cudaErrorInvalidValue;
-    }
+    if (Dp <= 32) SGM_MMA(32);
+    if (Dp <= 64) SGM_MMA(64);
+    SGM_MMA(128);
 #undef SGM_MMA
 }
 
@@ -468,7 +467,7 @@ cudaError_t launch_kb(const void *codes, int W, int H, int D, int nbits, uint8_t
 
 bool cost_mma_supported(int D) {
     const int Dp = padded_disparities(D);
-    return Dp == 32 || Dp == 64 || Dp == 128;
+    return Dp >= 32 && Dp <= 128;
 }
 
 cudaError_t launch_cost_mma(const void *codes, int code_bytes, int W, int H, int D, int nbits, uint8_t *cost,

@@ -281,7 +281,7 @@ sgm::ScratchSizes sgm::scratch_sizes(int W, int H, int D, const sgm_params *p) {
     const int nbits = p->census_w * p->census_h - 1;
     const size_t code_bytes = wide ? 0 : (nbits <= 32 ? 4 : 8);
     const size_t eb = wide ? 2 : 1;  // bytes per cost / path cost
-    const size_t npx = (size_t)W * H, Dp = (size_t)padded_disparities(D);
+    const size_t npx = (size_t)W * H, Dp = (size_t)scratch_disparities(D);
     const size_t npaths = (size_t)__builtin_popcount((unsigned)p->path_mask);
     ScratchSizes s;
     s.codes = 2 * npx * code_bytes;
