@@ -329,12 +329,12 @@ __device__ __forceinline__ Blk<NP, WIDE> path_step(PathState<NP> &st, const Blk<
     } else {
         // (m, m) = m * 0x10001 is monotonic in m; the other scanlines' lanes feed
         // x + 0x80008000, more than any (m, m)
-        mn = 0u;
+        uint32_t r[G];
 #pragma unroll
-        for (int g = 0; g < G; g++) {
-            const uint32_t r = __reduce_min_sync(0xffffffffu, mad(x, one, lg.grp == g ? 0u : 0x80008000u));
-            if (lg.grp == g) mn = r;
-        }
+        for (int g = 0; g < G; g++) r[g] = __reduce_min_sync(0xffffffffu, mad(x, one, lg.grp == g ? 0u : 0x80008000u));
+        if constexpr (G == 4) mn = lg.grp < 2 ? (lg.grp == 0 ? r[0] : r[1]) : (lg.grp == 2 ? r[2] : r[3]);
+        else mn = lg.grp == 0 ? r[0] : r[1];
+        static_assert(G == 2 || G == 4, "scanlines per warp that reduce with redux.sync");
     }
     st.m2 = mn;
     st.mQ = mad(mn, one, QPx2);
@@ -396,9 +396,9 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     lg.src_dn = last ? lane : lane + 1;
     lg.sel_dn = last ? 0x5476u : 0x3210u;
     lg.lo_mark = lg.first ? 0x7FFF7FFFu : 0u;
-    const int s = s0 + lg.grp;
-    int x = 0, y = 0, len = 0;
-    if (s < nlines) line_start(dx, dy, s, W, H, x, y, len);
+    // Likewise scanlines beyond the last repeat it.
+    int x, y, len;
+    line_start(dx, dy, min(s0 + lg.grp, nlines - 1), W, H, x, y, len);
     const int steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
     const int minlen = (int)__reduce_min_sync(0xffffffffu, (unsigned)len);
     // block indices: cost block (x, y, li) is cost[(y*W + x)*LPS + li], plane
@@ -421,10 +421,9 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     for (int p = 0; p < RT::kParts; p++) {
         const int unit = (p * 32 + lane) * RT::kCopy % RT::kStep;  // byte of the step
         const int cgrp = unit / rec;
-        int cx = 0, cy = 0;
-        clen[p] = 0;
+        int cx, cy;
+        line_start(dx, dy, min(s0 + cgrp, nlines - 1), W, H, cx, cy, clen[p]);
         mine[p] = FULL || cgrp < G;
-        if (mine[p] && s0 + cgrp < nlines) line_start(dx, dy, s0 + cgrp, W, H, cx, cy, clen[p]);
         ci[p] = (uint32_t)((((long long)cy * W + cx + csub * dir) * rec + (unit - cgrp * rec)) / RT::kCopy);
     }
     const uint32_t cadv = (uint32_t)(dir * RT::kPer * rec / RT::kCopy);
@@ -441,7 +440,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
             for (int p = 0; p < RT::kParts; p++) {
                 const uint32_t to = at + i * RT::kStep + p * 32 * RT::kCopy;
                 if constexpr (decltype(checked)::value) {
-                    const bool ok = blk * RT::kBlock + i + csub < clen[p] && in_range(ci[p], cost_copies);
+                    const bool ok = mine[p] && blk * RT::kBlock + i + csub < clen[p] && in_range(ci[p], cost_copies);
                     copy_or_zero<RT::kCopy>(to, cost + (ok ? ci[p] : 0u), ok);
                 } else if (mine[p] && in_range(ci[p], cost_copies)) {
                     copy_async<RT::kCopy>(to, cost + ci[p]);
@@ -484,18 +483,28 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
             cur = nxt;
         }
     }
+    // The blocks in which some scanline ends, a few steps at a time: what a
+    // scanline computes past its end is not stored.
+    constexpr int kTail = B < 4 ? B : 4;
+    static_assert(B % kTail == 0, "whole parts of a block");
 #pragma unroll 1
     for (; blk * B < steps; blk++) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
         __syncwarp();
         fetch(blk + kStages - 1, Checked());
         const uint32_t at = ring_r + (uint32_t)(blk % kStages) * RT::kBytes;
-        const int left = min(steps - blk * B, B);
 #pragma unroll 1
-        for (int i = 0; i < left; i++) {
-            const BT o = path_step<NP, G, WIDE>(st, ld_ring<NP, WIDE>(at + i * RT::kStep), P1x2, QPx2, lg, one);
-            if (blk * B + i < len && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
-            oi += ostep;
+        for (int i = 0; i < B && blk * B + i < steps; i += kTail) {
+            const int left = len - blk * B - i;
+            BT in[kTail];
+#pragma unroll
+            for (int q = 0; q < kTail; q++) in[q] = ld_ring<NP, WIDE>(at + (i + q) * RT::kStep);
+#pragma unroll
+            for (int q = 0; q < kTail; q++) {
+                const BT o = path_step<NP, G, WIDE>(st, in[q], P1x2, QPx2, lg, one);
+                if (q < left && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
+                oi += ostep;
+            }
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
