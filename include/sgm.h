@@ -240,9 +240,10 @@ int sgm_batch_device_bytes(sgm_batch b, size_t *bytes);
  * launched than there is work for) and disparities per lane, counted in chunks
  * of 8: 1 (the default), 2 or 4, or SGM_AGG_CHUNKS_MIXED.  With 1 a lane holds
  * one chunk, or half of one on the long-axis scanlines (rows when W >= H) while
- * D <= 128, whose chain of steps sets the kernel's duration; with 2 and 4 it
- * holds that many chunks in every direction; MIXED is one chunk on the
- * long-axis scanlines and two in the other directions.
+ * D <= 128, whose chain of steps sets the kernel's duration, and down to a
+ * quarter of one on small images; with 2 and 4 it holds that many chunks in
+ * every direction, and MIXED is one chunk on the long-axis scanlines and two
+ * in the other directions (where D spans a power of two of chunks; else as 1).
  * SGM_ERR_UNSUPPORTED above what D allows (D must span at least that many
  * chunks; the 16-bit costs of SGM_COST_SAD take 1).  More disparities per lane
  * let a warp walk more scanlines at once with fewer instructions per

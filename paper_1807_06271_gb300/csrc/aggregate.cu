@@ -41,9 +41,9 @@
 // Lanes per scanline.  One step of a scanline is a dependent chain: the update,
 // the minimum over the lanes, the next update.  Fewer disparities per lane
 // shorten it, more of them need fewer instructions per disparity.  The
-// long-axis scanlines (rows when W >= H) set the kernel's duration, so they
+// long-axis scanlines (rows when W >= H) are the longest chains, so they
 // run with 2 pairs per lane (a scanline of D = 128 fills a warp) and the other
-// directions with 4.
+// directions with 4; see lane_config for small images.
 //
 // Pipes.  On GB300 the packed minima, byte-permutes, logic, redux.sync and
 // three-input adds issue on the ALU pipe at 16 lanes per cycle (measured: 2
@@ -67,19 +67,56 @@
 
 namespace sgm {
 
-LaneConfig lane_config(int D, bool wide, int cpl) {
+namespace {
+
+constexpr int kSchedulers = 608;  // warp schedulers of the GPU (152 SMs)
+
+// Pairs per lane for a W x H image.  The base is 2 on the long axis and 4 in the
+// other directions (4 and 4 above D = 128).  Small images leave schedulers idle
+// and take as long as their longest chain of steps, so they get narrower lanes
+// (a step of one pair per lane and one scanline per warp takes 28 ns, of two and
+// two 40, of four and four 80; with D = 128, two and one 31, four and two 50).
+// Measured, aggregation in us:
+//   640 x 360, D = 60, 4 paths: base 37.6, (1, 4) 35.7, (1, 2) 32.8;  SAD 41.2, 38.6, 33.2
+//   640 x 480, D = 64, 4 paths: base 45.8, (1, 2) 39.1;  8 paths: base 69.4, (1, 2) 67.8, (2, 2) 61.3
+//   464 x 161, D = 64, 8 paths: base 28.8, (1, 4) 24.3, (1, 2) 28.0
+//   1280 x 720, D = 64, 8 paths: base 173.9, (1, 2) 176.4, (2, 2) 171.2
+//   320 x 240, D = 32, 4 paths: base 22.7, (1, 4) 22.8, (1, 1) 18.3;  1280 x 720, 8 paths: base 123.9, (1, 4) 132.9
+//   320 x 240, D = 128, 8 paths: base 35.0, (2, 2) 30.9;  480 x 752, 8 paths: base 102.8, (2, 2) 107.0
+LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool many) {
     const int Dp = padded_disparities(D);
     const bool pow2 = (Dp & (Dp - 1)) == 0;  // lanes of more than 4 pairs come in powers of two
     if (!wide && pow2 && cpl == 2) return {8, 8};
     if (!wide && pow2 && cpl == 4) return {16, 16};
     if (!wide && pow2 && cpl == kMixedCpl) return {4, 8};
-    return {Dp <= 128 ? 2 : 4, 4};
+    LaneConfig lc{Dp <= 128 ? 2 : 4, 4};
+    if (many || Dp < 32 || Dp > 128) return lc;
+    const int axis = W >= H ? 0x03 : 0x0C;  // the long-axis directions
+    long lines_long = 0, lines_other = 0;
+    for (int r = 0; r < kMaxPaths; r++)
+        if ((mask >> r) & 1) (((axis >> r) & 1) ? lines_long : lines_other) += scanlines_of(r, W, H);
+    auto warps = [&](int np_long, int np_other) {
+        return lines_long * lanes_of(D, np_long) / 32 + lines_other * lanes_of(D, np_other) / 32;
+    };
+    if (Dp == 32) {
+        if (warps(1, 1) <= 2 * kSchedulers) return {1, 1};
+        if (warps(1, 4) <= 3 * kSchedulers) return {1, 4};
+        return lc;
+    }
+    // narrower lanes in the other directions where their chain is the longer one
+    const double chain_long = (Dp == 64 ? 28. : 31.) * (W >= H ? W : H), chain_other = (Dp == 64 ? 80. : 50.) * (W >= H ? H : W);
+    if (chain_other > chain_long && warps(2, 2) <= 12 * kSchedulers) lc.np_other = 2;
+    if (Dp == 64 && warps(1, lc.np_other) <= 3 * kSchedulers) lc.np_long = 1;
+    return lc;
 }
 
-PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl) {
+}  // namespace
+
+PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool many) {
     PathJobs j = {};
     j.unit = 1u;
-    const LaneConfig lc = lane_config(D, wide, cpl);
+    const LaneConfig lc = lane_config(W, H, D, mask, wide, cpl, many);
+    j.lanes = lc;
     // long axis first, then the short axis, then the diagonals; each entry is a
     // direction and its opposite
     const int first[4] = {W >= H ? 0 : 2, W >= H ? 2 : 0, 4, 6};
@@ -152,10 +189,13 @@ __device__ __forceinline__ int next_job(unsigned *counter, int total, int lane) 
 }
 
 // The NP pairs one lane holds, as they sit in the cost volume and the planes:
-// 2 bytes per pair for 8-bit costs, 4 for the 16-bit costs of SAD.
+// 2 bytes per pair for 8-bit costs, 4 for the 16-bit costs of SAD.  With one
+// 8-bit pair per lane (kHalf) two lanes share a word; the even one stores it.
 template <int NP, bool WIDE>
 struct Blk {
-    static constexpr int kWords = WIDE ? NP : NP / 2;
+    static constexpr bool kHalf = NP == 1 && !WIDE;
+    static constexpr int kLane = WIDE ? 4 * NP : 2 * NP;  // bytes of a lane
+    static constexpr int kWords = WIDE ? NP : NP == 1 ? 1 : NP / 2;
     static_assert(kWords == 1 || kWords == 2 || kWords % 4 == 0, "a lane block is 4, 8 or whole 16-byte vectors");
     uint32_t w[kWords];
 };
@@ -200,12 +240,12 @@ __device__ __forceinline__ void st_blk(Blk<NP, WIDE> *p, const Blk<NP, WIDE> &v,
 // warp moves kCopy bytes per lane, kPer steps together (or a part of one).
 template <int NP, int G, bool WIDE>
 struct Ring {
-    static constexpr int kStep = 32 * 4 * Blk<NP, WIDE>::kWords;  // bytes of a step
-    static constexpr bool kTiny = G >= 8 && (32 / G) * 4 * Blk<NP, WIDE>::kWords == 8;  // records of 8 bytes
+    static constexpr int kStep = 32 * Blk<NP, WIDE>::kLane;                           // bytes of a step
+    static constexpr bool kTiny = G >= 8 && (32 / G) * Blk<NP, WIDE>::kLane == 8;  // records of 8 bytes
     static constexpr int kCopy = kTiny ? 8 : 16;
     static constexpr int kPer = 32 * kCopy >= kStep ? 32 * kCopy / kStep : 1;     // steps of a copy
     static constexpr int kParts = 32 * kCopy >= kStep ? 1 : kStep / (32 * kCopy);  // copies of a step
-    static constexpr int kBlock = (kRingBytes / kStages) / kStep;   // steps of a stage
+    static constexpr int kBlock = kRingBytes / kStages / kStep < 16 ? kRingBytes / kStages / kStep : 16;  // steps of a stage
     static constexpr int kBytes = kBlock * kStep;
     static_assert(kStages * kBytes <= kRingBytes, "the ring holds the stages");
 };
@@ -230,6 +270,7 @@ struct LaneGeom {
     int grp, li;          // scanline of the warp, lane within it
     int src_up, src_dn;   // lanes that hold the neighbouring pairs (its own at the scanline's ends)
     uint32_t sel_dn;      // byte-permute selector: the lane after, or its own last pair swapped
+    uint32_t sel_c;       // byte-permute selector of a lane's pair in the word it shares
     uint32_t lo_mark;     // added to the pair before the scanline's first one
     bool first;
 };
@@ -263,7 +304,9 @@ __device__ __forceinline__ Blk<NP, WIDE> path_step(PathState<NP> &st, const Blk<
     for (int w = 0; w < NP; w += 2) {
         if constexpr (WIDE) {
             c[w] = b.w[w];
-            c[w + 1] = b.w[w + 1];
+            if (NP > 1) c[NP > 1 ? w + 1 : 0] = b.w[NP > 1 ? w + 1 : 0];
+        } else if constexpr (NP == 1) {
+            c[0] = __byte_perm(b.w[0], 0u, lg.sel_c);
         } else {
             const uint32_t v = b.w[w / 2];
             c[w] = __byte_perm(v, 0u, 0x4341);               // bytes 1, 3
@@ -279,7 +322,8 @@ __device__ __forceinline__ Blk<NP, WIDE> path_step(PathState<NP> &st, const Blk<
         const uint32_t dn = __shfl_sync(0xffffffffu, st.R[0], lg.src_dn);
         after = __byte_perm(dn, st.R[NP - 1], lg.sel_dn);
         // the first lane got its own last pair: for NP = 2 that is a neighbour of
-        // its first pair anyway; otherwise it is lifted out of the way
+        // its first pair anyway, for NP = 1 the pair itself, which changes nothing;
+        // otherwise it is lifted out of the way
         if constexpr (NP > 2) {
             if constexpr (WIDE) before = lg.first ? st.R[1] : before;
             else before = mad(before, one, lg.lo_mark);
@@ -297,6 +341,8 @@ __device__ __forceinline__ Blk<NP, WIDE> path_step(PathState<NP> &st, const Blk<
     if constexpr (WIDE) {
 #pragma unroll
         for (int k = 0; k < NP; k++) out.w[k] = n[k];
+    } else if constexpr (NP == 1) {
+        out.w[0] = mad(n[0], one * 256u, __shfl_xor_sync(0xffffffffu, n[0], 1));  // of even lanes
     } else if constexpr (kTiny) {
 #pragma unroll
         for (int w = 0; w < NP / 2; w++) out.w[w] = __byte_perm(n[2 * w + 1], n[2 * w], 0x6240);
@@ -310,7 +356,7 @@ __device__ __forceinline__ Blk<NP, WIDE> path_step(PathState<NP> &st, const Blk<
     uint32_t x = n[0];
     if constexpr (NP == 2) {
         x = vmin2(n[0], n[1]);
-    } else {
+    } else if constexpr (NP > 2) {
         uint32_t y = __vimin3_u16x2(n[0], n[1], n[2]);
 #pragma unroll
         for (int k = 3; k + 1 < NP; k += 2) y = __vimin3_u16x2(y, n[k], n[k + 1]);
@@ -396,6 +442,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     lg.src_dn = last ? lane : lane + 1;
     lg.sel_dn = last ? 0x5476u : 0x3210u;
     lg.lo_mark = lg.first ? 0x7FFF7FFFu : 0u;
+    lg.sel_c = lg.li & 1 ? 0x4240u : 0x4341u;
     // Likewise scanlines beyond the last repeat it.
     int x, y, len;
     line_start(dx, dy, min(s0 + lg.grp, nlines - 1), W, H, x, y, len);
@@ -405,14 +452,16 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     // block is planes[((y*W + x)*nplanes + plane)*LPS + li] (all planes of a
     // pixel are adjacent).  They stay below 2^32 (checked at handle creation).
     const long long pix = (long long)y * W + x, dir = (long long)dy * W + dx;
-    const long long cost_copies = (long long)W * H * LPS * (int)sizeof(BT) / RT::kCopy, plane_blocks = (long long)W * H * LPS * nplanes;
+    const int rec = LPS * BT::kLane;  // bytes of a pixel's record
+    const long long cost_copies = (long long)W * H * rec / RT::kCopy;
+    const long long plane_blocks = (long long)W * H * nplanes * rec / (int)sizeof(BT);
     // the lane block of the step to store (their count stays below 2^32, checked at
     // handle creation; 32 bits keep the address arithmetic on the FMA pipe)
-    uint32_t oi = (uint32_t)((pix * nplanes + plane) * LPS + lg.li);
-    const uint32_t ostep = (uint32_t)(dir * nplanes * LPS);
+    uint32_t oi = (uint32_t)(((pix * nplanes + plane) * rec + lg.li * BT::kLane) / (int)sizeof(BT));
+    const uint32_t ostep = (uint32_t)(dir * nplanes * rec / (int)sizeof(BT));
+    const bool stores = !BT::kHalf || !(lg.li & 1);
     // this lane's share of the copies: kCopy bytes at offset ccol of the record of
     // scanline s0 + cgrp (one per part of a step), csub steps into the copy
-    const int rec = LPS * (int)sizeof(BT);  // bytes of a pixel's record
     const int csub = lane * RT::kCopy / RT::kStep;
     int clen[RT::kParts];
     bool mine[RT::kParts];  // a step's records may be shorter than the warp's copies
@@ -427,7 +476,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
         ci[p] = (uint32_t)((((long long)cy * W + cx + csub * dir) * rec + (unit - cgrp * rec)) / RT::kCopy);
     }
     const uint32_t cadv = (uint32_t)(dir * RT::kPer * rec / RT::kCopy);
-    const uint32_t ring_w = ring + lane * RT::kCopy, ring_r = ring + vl * (int)sizeof(BT);
+    const uint32_t ring_w = ring + lane * RT::kCopy, ring_r = ring + (vl * BT::kLane & ~3);
     using CT = typename std::conditional<RT::kCopy == 16, uint4, uint2>::type;
     const CT *__restrict__ cost = reinterpret_cast<const CT *>(cost_);
     BT *__restrict__ planes = reinterpret_cast<BT *>(planes_);
@@ -478,7 +527,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
             BT nxt = cur;
             if (i + 1 < B) nxt = ld_ring<NP, WIDE>(at + (i + 1) * RT::kStep);
             const BT o = path_step<NP, G, WIDE>(st, cur, P1x2, QPx2, lg, one);
-            if (in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
+            if (stores && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
             oi += ostep;
             cur = nxt;
         }
@@ -502,7 +551,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
 #pragma unroll
             for (int q = 0; q < kTail; q++) {
                 const BT o = path_step<NP, G, WIDE>(st, in[q], P1x2, QPx2, lg, one);
-                if (q < left && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
+                if (stores && q < left && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
                 oi += ostep;
             }
         }
@@ -513,7 +562,7 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
 // Jobs of the long-axis entry hold NPL pairs per lane (GL scanlines per warp),
 // the others NPO (GO).
 template <int NPL, int GL, int NPO, int GO, bool WIDE, bool FULL>
-__global__ void __launch_bounds__(kWarps * 32, 5)
+__global__ void __launch_bounds__(kWarps * 32, 6)
     aggregate_kernel(const void *__restrict__ cost, int W, int H, int Dp, uint32_t P1x2, uint32_t P2x2,
                      const __grid_constant__ PathJobs jobs, void *__restrict__ planes, int nplanes,
                      unsigned *__restrict__ job_counter, int sms) {
@@ -546,7 +595,7 @@ __host__ __device__ constexpr int lines_per_warp(int Dp, int np) { return Dp / (
 // pfx[0][p] and pfx[1][p].  Each job runs with its pair's lanes per scanline;
 // CPL == 4 adds the lanes of 16 pairs.
 template <int CPL, bool WIDE>
-__global__ void __launch_bounds__(kWarps * 32, 5)
+__global__ void __launch_bounds__(kWarps * 32, 6)
     aggregate_batch_kernel(const BatchAggPair *__restrict__ pairs, int npairs, const int *__restrict__ prefix,
                            uint32_t P1x2, uint32_t P2x2, unsigned *__restrict__ job_counter, int sms) {
     wait_for_predecessor();
@@ -583,7 +632,7 @@ __global__ void __launch_bounds__(kWarps * 32, 5)
                                  p.jobs.unit);
         };
         // pairs per lane of this job, and scanlines per warp
-        const int np = lq ? p.np_long : p.np_other;
+        const int np = lq ? p.jobs.lanes.np_long : p.jobs.lanes.np_other;
 #define SGM_JOB(NP, G) \
     case 64 * NP + G: job_as(std::integral_constant<int, NP>(), std::integral_constant<int, G>()); break
         switch (64 * np + lines_per_warp(p.Dp, np)) {
@@ -624,11 +673,18 @@ AggKernel agg_kernel_t(int Dp, LaneConfig lc) {
     SGM_AGG(2, 16, 4, 32);  // Dp = 8
     SGM_AGG(2, 8, 4, 16);   // 16
     SGM_AGG(2, 4, 4, 8);    // 32
+    SGM_AGG(1, 2, 4, 8);
+    SGM_AGG(1, 2, 1, 2);
     SGM_AGG(2, 2, 4, 4);    // 64
-    SGM_AGG(2, 1, 4, 2);    // 128
-    SGM_AGG(4, 1, 4, 1);    // 256
+    SGM_AGG(2, 2, 2, 2);
+    SGM_AGG(1, 1, 4, 4);
+    SGM_AGG(1, 1, 2, 2);
     SGM_AGG_F(2, 1, 4, 2, false);  // 96
+    SGM_AGG_F(2, 1, 2, 1, false);
+    SGM_AGG(2, 1, 4, 2);    // 128
+    SGM_AGG(2, 1, 2, 1);
     SGM_AGG_F(4, 1, 4, 1, false);  // 160, 192, 224
+    SGM_AGG(4, 1, 4, 1);    // 256
     if constexpr (!WIDE) {  // Dp a power of two, 16 to 256
         SGM_AGG(8, 32, 8, 32);
         SGM_AGG(8, 16, 8, 16);
@@ -692,7 +748,7 @@ cudaError_t launch_aggregate(const uint8_t *cost, int W, int H, int D, int P1, i
     const int wanted = sms * (blocks_per_sm > 0 ? blocks_per_sm : 2), filled = (jobs.jbegin[jobs.n] + kWarps - 1) / kWarps;
     const int blocks = filled < sms ? sms : filled < wanted ? filled : wanted;
     const int Dp = padded_disparities(D);
-    const LaneConfig lc = lane_config(D, wide, cpl);
+    const LaneConfig lc = jobs.lanes;
     const uint32_t P1x2 = (uint32_t)P1 * 0x00010001u, P2x2 = (uint32_t)P2 * 0x00010001u;
     auto kernel = agg_kernel(Dp, lc, wide);
     if (!kernel) return cudaErrorInvalidValue;

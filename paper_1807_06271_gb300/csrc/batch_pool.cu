@@ -130,11 +130,8 @@ int layout_groups(sgm_batch_s *b, int ng, bool upload, size_t at, size_t *end) {
             t.W = ps.W;
             t.H = ps.H;
             t.Dp = ps.Dp;
-            const LaneConfig lc = lane_config(ps.D, b->wide != 0, b->cpl);
-            t.np_long = lc.np_long;
-            t.np_other = lc.np_other;
             t.nplanes = b->npaths;
-            t.jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl);
+            t.jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl, b->n > 1);
             prefix[k + 1] = prefix[k] + t.jobs.nlong;
             prefix[np + 1 + k + 1] = prefix[np + 1 + k] + (t.jobs.jbegin[t.jobs.n] - t.jobs.nlong);
         }
@@ -212,7 +209,7 @@ int enqueue(sgm_batch_s *b, const uint8_t *const *left, const uint8_t *const *ri
             // (overlapped) dependency on the one before it.
             const int i = g.pairs[0];
             PairSlot &ps = b->pairs[i];
-            const PathJobs jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl);
+            const PathJobs jobs = make_path_jobs(ps.W, ps.H, ps.D, b->p.path_mask, b->wide != 0, b->cpl, b->n > 1);
             if (costs(i, job_state) != cudaSuccess ||
                 launch_aggregate(b->pool + ps.cost, ps.W, ps.H, ps.D, b->p.P1, b->p.P2, b->wide != 0, jobs,
                                  b->pool + ps.planes, b->npaths, job_state, b->blocks_per_sm, b->cpl,

@@ -144,12 +144,10 @@ constexpr unsigned kPadCost = 255u, kPadCostWide = 0x7FFFu;
 constexpr bool kPlanar = false;
 
 // Pairs of disparities a lane of the aggregation kernel holds, for the
-// long-axis scanlines and for the other directions, under the
-// sgm_set_aggregation setting cpl.
+// long-axis scanlines and for the other directions.
 struct LaneConfig {
     int np_long, np_other;
 };
-LaneConfig lane_config(int D, bool wide, int cpl);
 inline int lanes_of(int D, int np) { return padded_disparities(D) / (2 * np); }
 
 // Work list of the aggregation kernel: entry k is one enabled direction, or a
@@ -158,6 +156,7 @@ inline int lanes_of(int D, int np) { return padded_disparities(D) / (2 * np); }
 // of the two directions alternate.  Job j belongs to entry k when jbegin[k] <=
 // j < jbegin[k+1].
 struct PathJobs {
+    LaneConfig lanes;
     int n;                       // number of entries
     int ndir[kMaxPaths / 2];     // directions of entry k
     int dx[kMaxPaths / 2][2], dy[kMaxPaths / 2][2];
@@ -173,8 +172,10 @@ struct PathJobs {
 constexpr size_t kJobStateBytes = 4224;
 
 // Builds the work list for the directions in `mask` (planes numbered in
-// increasing direction order), longest scanlines first.
-PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl);
+// increasing direction order), longest scanlines first, under the
+// sgm_set_aggregation setting cpl.  many: other pairs' work runs beside it, so
+// the lanes are not narrowed to shorten a small image's chains.
+PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool many = false);
 // The most chunks per lane the aggregation takes for D (1 for 16-bit costs, up to 4).
 int chunks_per_lane_max(int D, bool wide);
 // Chunks-per-lane code of the mixed layout: long-axis scanlines at 1, the others at 2.
@@ -184,7 +185,7 @@ constexpr int kMixedCpl = SGM_AGG_CHUNKS_MIXED;
 struct BatchAggPair {
     const void *cost;  // the pair's cost volume
     void *planes;      // its path planes
-    int W, H, Dp, np_long, np_other;
+    int W, H, Dp;
     int nplanes;
     PathJobs jobs;
 };
