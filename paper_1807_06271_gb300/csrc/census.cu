@@ -310,8 +310,6 @@ cudaError_t launch_cost(const void *codes, int code_bytes, int W, int H, int D, 
     const size_t smem = (((size_t)kSeg * (Dp + 8) + 15) & ~(size_t)15) + (size_t)(2 * kSeg + Dp + 2) * code_bytes;
     const dim3 grid((W + kSeg - 1) / kSeg, H);
     auto go = [&](auto kernel, auto *c) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         return launch_k(kernel, grid, dim3(kCostThreads), smem, s, c, W, H, D, Dp, nbits, cost, job_state);
     };
     const bool rag = D != Dp;

@@ -172,13 +172,34 @@ def _check(rc: int, what: str):
         raise SgmError(rc, what)
 
 
+# The calls on small images are as fast as the host issues them, so the two
+# helpers below stay off torch's slow paths (measured on the Grace host, per
+# call: the current stream 3.0 -> 0.2 us, a buffer check 0.53 -> 0.44).
+_raw_stream = None  # the current stream of the current device, as a cudaStream_t
+
+
+def _make_raw_stream():
+    import torch
+    try:
+        get_stream, get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    except AttributeError:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    torch.cuda.current_stream()  # initialises CUDA as it always did
+    return lambda: get_stream(get_device())
+
+
 def _stream(stream):
+    global _raw_stream
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _raw_stream is None:
+            _raw_stream = _make_raw_stream()
+        return _raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+_dtype_ok = {}  # (dtype, accepted names) -> whether the dtype is one of them
 
 
 def _dev(t, dtype_names, shape, what):
@@ -187,13 +208,22 @@ def _dev(t, dtype_names, shape, what):
         return None
     if not t.is_cuda:
         raise ValueError(f"{what}: expected a CUDA tensor")
-    if str(t.dtype).replace("torch.", "") not in dtype_names:
+    key = (t.dtype, dtype_names)
+    ok = _dtype_ok.get(key)
+    if ok is None:
+        ok = _dtype_ok[key] = str(t.dtype).replace("torch.", "") in dtype_names
+    if not ok:
         raise ValueError(f"{what}: dtype {t.dtype} not in {dtype_names}")
     if not t.is_contiguous():
         raise ValueError(f"{what}: tensor must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape and tuple(t.shape) != tuple(shape):
         raise ValueError(f"{what}: shape {tuple(t.shape)} != {tuple(shape)}")
     return t.data_ptr()
+
+
+_U8 = ("uint8",)
+_U16 = ("uint16", "int16")
+_Int4 = ctypes.c_int * 4
 
 
 class Handle:
@@ -253,16 +283,15 @@ def sgm_destroy(h):
 
 def sgm_compute(h: Handle, left, right, disp, stream=None):
     shp = h._img_shape()
-    _check(load().sgm_compute(
-        h.ptr, _dev(left, ("uint8",), shp, "left"), _dev(right, ("uint8",), shp, "right"),
-        _dev(disp, ("uint8",), (h.H, h.W), "disp"), _stream(stream)), "sgm_compute")
+    _check((_lib or load()).sgm_compute(
+        h.ptr, _dev(left, _U8, shp, "left"), _dev(right, _U8, shp, "right"),
+        _dev(disp, _U8, (h.H, h.W), "disp"), _stream(stream)), "sgm_compute")
 
 
 def uvmap_compute(h: Handle, disp, umap, vmap, stream=None):
-    _check(load().uvmap_compute(
-        h.ptr, _dev(disp, ("uint8",), (h.H, h.W), "disp"),
-        _dev(umap, ("uint16", "int16"), (h.D, h.W), "umap"),
-        _dev(vmap, ("uint16", "int16"), (h.H, h.D), "vmap"), _stream(stream)), "uvmap_compute")
+    _check((_lib or load()).uvmap_compute(
+        h.ptr, _dev(disp, _U8, (h.H, h.W), "disp"), _dev(umap, _U16, (h.D, h.W), "umap"),
+        _dev(vmap, _U16, (h.H, h.D), "vmap"), _stream(stream)), "uvmap_compute")
 
 
 def _host(t, nbytes, what):
@@ -607,12 +636,10 @@ def uvmap_postprocess(h: Handle, umap, vmap, u_threshold: int, v_threshold: int,
     """Thresholded, dilated and Gaussian-smoothed U-/V-maps (uint8) of Sec. 3.2."""
     u_roi = u_roi or (0, h.D, 0, h.W)
     v_roi = v_roi or (0, h.H, 0, h.D)
-    p = _UvPost(u_threshold, v_threshold, (ctypes.c_int * 4)(*u_roi), (ctypes.c_int * 4)(*v_roi),
-                dilate_r)
-    _check(load().uvmap_postprocess(
-        h.ptr, _dev(umap, ("uint16", "int16"), (h.D, h.W), "umap"),
-        _dev(vmap, ("uint16", "int16"), (h.H, h.D), "vmap"), ctypes.byref(p),
-        _dev(uout, ("uint8",), (h.D, h.W), "uout"), _dev(vout, ("uint8",), (h.H, h.D), "vout"),
+    p = _UvPost(u_threshold, v_threshold, _Int4(*u_roi), _Int4(*v_roi), dilate_r)
+    _check((_lib or load()).uvmap_postprocess(
+        h.ptr, _dev(umap, _U16, (h.D, h.W), "umap"), _dev(vmap, _U16, (h.H, h.D), "vmap"), ctypes.byref(p),
+        _dev(uout, _U8, (h.D, h.W), "uout"), _dev(vout, _U8, (h.H, h.D), "vout"),
         _stream(stream)), "uvmap_postprocess")
 
 
