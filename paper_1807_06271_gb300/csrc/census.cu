@@ -164,16 +164,19 @@ constexpr int kCostThreads = 64, kSeg = 32;
 __device__ __forceinline__ uint32_t popcnt(uint32_t v) { return __popc(v); }
 __device__ __forceinline__ uint32_t popcnt(uint64_t v) { return __popcll(v); }
 
-template <typename CodeT, bool RAGGED>
+// Dp is a template parameter: with it at run time the loops' address and piece
+// arithmetic took a fifth of the instructions (1280 x 720, D = 128, 24-bit codes: 45.0
+// us; pieces stepped without a division 41.1; this 33.0).
+template <typename CodeT, int Dp, bool RAGGED>
 __global__ void __launch_bounds__(kCostThreads)
-    cost_kernel(const CodeT *__restrict__ codes, int W, int H, int D, int Dp, int nbits,
-                uint8_t *__restrict__ cost, unsigned *__restrict__ job_state) {
+    cost_kernel(const CodeT *__restrict__ codes, int W, int H, int D, int nbits, uint8_t *__restrict__ cost,
+                unsigned *__restrict__ job_state) {
     wait_for_predecessor();
     if (job_state && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *job_state = 0u;
     extern __shared__ __align__(16) unsigned char cost_smem[];
-    const int stride = Dp + 8;  // padded tile row (bytes)
+    constexpr int stride = Dp + 8;  // padded tile row (bytes)
     uint8_t *tile = cost_smem;                                          // [kSeg][stride]
-    const int tile_bytes = (kSeg * stride + 15) & ~15;
+    constexpr int tile_bytes = (kSeg * stride + 15) & ~15;
     CodeT *cl = reinterpret_cast<CodeT *>(cost_smem + tile_bytes);     // [kSeg]
     CodeT *cr = cl + kSeg;                                              // [kSeg + Dp + 2]
     const int y = blockIdx.y, x0 = blockIdx.x * kSeg;
@@ -187,7 +190,7 @@ __global__ void __launch_bounds__(kCostThreads)
         cr[i] = (xr >= 0 && xr < W && in_range((long long)W * H + (long long)y * W + xr, 2LL * W * H)) ? rowr[xr] : 0;
     }
     __syncthreads();
-    const int chunks = Dp / 8;
+    constexpr int chunks = Dp / 8;
     const bool border = x0 < Dp;  // only the first segments see x - d < 0
     // A thread takes the two words (four pairs) i of the pixel pair (px, px+1), px
     // even: the disparities 4i + e and Dp-1-4i-e, e < 4.  Column x - d of pixel px
@@ -212,8 +215,8 @@ __global__ void __launch_bounds__(kCostThreads)
     };
     CodeT a0, a1;
     two(cl + px, a0, a1);
-    for (int it = threadIdx.x; it < (kSeg / 2) * chunks; it += kCostThreads) {
-        const int i = it / (kSeg / 2);
+#pragma unroll 2
+    for (int i = threadIdx.x / (kSeg / 2); i < chunks; i += kCostThreads / (kSeg / 2)) {
         const CodeT *rl = cr + px + Dp - 2 - 4 * i, *rh = cr + px + 2 + 4 * i;
         CodeT wl[5], wh[5];
         two(rl, wl[0], wl[1]);
@@ -251,13 +254,21 @@ __global__ void __launch_bounds__(kCostThreads)
     __syncthreads();
     const int npx = min(kSeg, W - x0);
     uint8_t *out = cost + ((size_t)y * W + x0) * Dp;
-    for (int k = threadIdx.x; k < npx * chunks; k += kCostThreads) {
-        const int px = k / chunks, q = k - px * chunks;
+    // thread t copies the 8-byte pieces t, t + kCostThreads, ..: piece q of pixel p,
+    // stepped along without a division per piece
+    constexpr int dp = kCostThreads / chunks, dq = kCostThreads - dp * chunks;
+    int p = threadIdx.x / chunks, q = threadIdx.x - p * chunks;
+    while (p < npx) {
         // a record of 8 bytes starting at byte o of the W x H x Dp volume
-        const long long o = ((long long)y * W + x0 + px) * Dp + 8 * q;
+        const long long o = ((long long)y * W + x0 + p) * Dp + 8 * q;
         if (in_range(o, (long long)W * H * Dp - 8 + 1))
-            *reinterpret_cast<uint2 *>(out + (size_t)px * Dp + 8 * q) =
-                *reinterpret_cast<const uint2 *>(tile + px * stride + 8 * q);
+            *reinterpret_cast<uint2 *>(out + p * Dp + 8 * q) = *reinterpret_cast<const uint2 *>(tile + p * stride + 8 * q);
+        p += dp;
+        q += dq;
+        if (q >= chunks) {
+            q -= chunks;
+            p++;
+        }
     }
 }
 
@@ -310,17 +321,31 @@ cudaError_t launch_cost(const void *codes, int code_bytes, int W, int H, int D, 
     const size_t smem = (((size_t)kSeg * (Dp + 8) + 15) & ~(size_t)15) + (size_t)(2 * kSeg + Dp + 2) * code_bytes;
     const dim3 grid((W + kSeg - 1) / kSeg, H);
     auto go = [&](auto kernel, auto *c) {
-        return launch_k(kernel, grid, dim3(kCostThreads), smem, s, c, W, H, D, Dp, nbits, cost, job_state);
+        return launch_k(kernel, grid, dim3(kCostThreads), smem, s, c, W, H, D, nbits, cost, job_state);
     };
     const bool rag = D != Dp;
+    const uint32_t *c4 = (const uint32_t *)codes;
+    const uint64_t *c8 = (const uint64_t *)codes;
     cudaError_t e;
-    if (code_bytes == 4) {
-        const uint32_t *c = (const uint32_t *)codes;
-        e = rag ? go(cost_kernel<uint32_t, true>, c) : go(cost_kernel<uint32_t, false>, c);
-    } else {
-        const uint64_t *c = (const uint64_t *)codes;
-        e = rag ? go(cost_kernel<uint64_t, true>, c) : go(cost_kernel<uint64_t, false>, c);
+#define SGM_COST(P)                                                                                       \
+    case P:                                                                                               \
+        if (code_bytes == 4) e = rag ? go(cost_kernel<uint32_t, P, true>, c4) : go(cost_kernel<uint32_t, P, false>, c4); \
+        else e = rag ? go(cost_kernel<uint64_t, P, true>, c8) : go(cost_kernel<uint64_t, P, false>, c8);                 \
+        break
+    switch (Dp) {
+        SGM_COST(8);
+        SGM_COST(16);
+        SGM_COST(32);
+        SGM_COST(64);
+        SGM_COST(96);
+        SGM_COST(128);
+        SGM_COST(160);
+        SGM_COST(192);
+        SGM_COST(224);
+        SGM_COST(256);
+        default: return cudaErrorInvalidValue;
     }
+#undef SGM_COST
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
