@@ -42,7 +42,12 @@ namespace {
 // SM) 80.2 / 77.5 / 16.9; 4 and 4 77.1 / 80.6 / 18.9 but 673 against 598 at 1920 x 1080.
 // A row split over a cluster of 2 or 4 CTAs that merge their minima at the end
 // measured 82-85 / 80-84.
-constexpr int kThreads = 512, kWarps = kThreads / 32;
+//
+// 16-bit records of 8 paths are 192 KB of ring at 16 warps, which leaves room for
+// rows of some 6900 pixels; longer ones halve the warps (wta_warps below).  Only
+// the kernels for any number of planes take the warps from the block size: the
+// others lose 5 % by it (80.1 -> 86.9 at 1242 x 375).
+constexpr int kMaxWarps = 16;
 constexpr int kStages = 3;
 
 // Minimum of v over the lanes of this lane's pixel (grp of the warp's G): one
@@ -78,9 +83,9 @@ __device__ __forceinline__ void copy8(uint32_t dst, const uint8_t *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 
-// NP > 0: NP planes (compile time); NP == 0: nplanes at run time.
+// NP > 0: NP planes and kMaxWarps warps (compile time); NP == 0: any of both.
 template <int G, bool WIDE, int NP, bool DEBUG>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kMaxWarps * 32)
     wta_kernel(const uint8_t *__restrict__ planes, int nplanes, int W, int H, int D, int Dp, int tol,
                uint8_t *__restrict__ disp_lr, uint8_t *__restrict__ dbg_left, uint8_t *__restrict__ dbg_right,
                uint16_t *__restrict__ dbg_sum) {
@@ -90,17 +95,18 @@ __global__ void __launch_bounds__(kThreads)
     const int np = NP > 0 ? NP : nplanes;
     const int rec = np * Dp * EB;  // bytes of a pixel's record
     const int lps = Dp / 8;        // lanes per pixel
+    const int warps = NP > 0 ? kMaxWarps : (int)blockDim.x / 32;
     extern __shared__ __align__(16) uint8_t wta_smem[];
-    uint8_t *ring = wta_smem;  // [kWarps][kStages][G][rec]
-    uint32_t *key_right = reinterpret_cast<uint32_t *>(wta_smem + (size_t)kWarps * kStages * G * rec);  // slots -Dp .. W-1
+    uint8_t *ring = wta_smem;  // [warps][kStages][G][rec]
+    uint32_t *key_right = reinterpret_cast<uint32_t *>(wta_smem + (size_t)warps * kStages * G * rec);  // slots -Dp .. W-1
     uint8_t *dl_row = reinterpret_cast<uint8_t *>(key_right + Dp + W);                                // W bytes
     const int y = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = lane / lps, li = lane - grp * lps;
-    for (int i = threadIdx.x; i < Dp + W; i += kThreads) key_right[i] = 0xFFFFFFFFu;
+    for (int i = threadIdx.x; i < Dp + W; i += warps * 32) key_right[i] = 0xFFFFFFFFu;
     __syncthreads();
     // this group's pixels [xb, xe); lanes past the last group have none
-    const int seg = (W + kWarps * G - 1) / (kWarps * G);
+    const int seg = (W + warps * G - 1) / (warps * G);
     const int xb = min((warp * G + grp) * seg, W), xe = grp < G ? min(xb + seg, W) : xb;
     const uint64_t pol = policy_evict_first();
     const uint32_t ring_warp = (uint32_t)__cvta_generic_to_shared(ring) + (uint32_t)(warp * kStages * G * rec);
@@ -227,7 +233,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    for (int xx = threadIdx.x; xx < W; xx += kThreads) {
+    for (int xx = threadIdx.x; xx < W; xx += warps * 32) {
         const int dl = dl_row[xx];
         uint8_t v = (uint8_t)dl;
         if (tol >= 0) {
@@ -248,23 +254,37 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
+// Shared memory of a CTA: the rings (rec bytes per warp and stage), the right minima
+// and the left winners of the row.
+size_t wta_smem_bytes(int W, int Dp, size_t rec, int warps) {
+    return (size_t)warps * kStages * rec + (size_t)(Dp + W) * sizeof(uint32_t) + (size_t)((W + 3) & ~3);
+}
+
+// As many warps as fit a CTA's 227 KB.
+int wta_warps(int W, int Dp, size_t rec) {
+    int warps = kMaxWarps;
+    while (warps > 1 && wta_smem_bytes(W, Dp, rec, warps) > 227 * 1024) warps /= 2;
+    return warps;
+}
+
 template <bool WIDE>
 cudaError_t launch_wta_t(const uint8_t *planes, int nplanes, int W, int H, int D, int tol, uint8_t *disp_lr,
                          uint8_t *dbg_left, uint8_t *dbg_right, uint16_t *dbg_sum, cudaStream_t s) {
     const int Dp = padded_disparities(D);
+    const int warps = wta_warps(W, Dp, (size_t)(256 / Dp) * nplanes * Dp * (WIDE ? 2 : 1));
+    const bool all = warps == kMaxWarps;
     auto go = [&](auto kernel, int G) {
-        const size_t smem = (size_t)kWarps * kStages * G * nplanes * Dp * (WIDE ? 2 : 1) +
-                            (size_t)(Dp + W) * sizeof(uint32_t) + (size_t)((W + 3) & ~3);
+        const size_t smem = wta_smem_bytes(W, Dp, (size_t)G * nplanes * Dp * (WIDE ? 2 : 1), warps);
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        return launch_k(kernel, dim3(H), dim3(kThreads), smem, s, planes, nplanes, W, H, D, Dp, tol, disp_lr, dbg_left,
+        return launch_k(kernel, dim3(H), dim3(warps * 32), smem, s, planes, nplanes, W, H, D, Dp, tol, disp_lr, dbg_left,
                         dbg_right, dbg_sum);
     };
-#define SGM_WTA(G)                                                         \
-    case G:                                                                \
-        if (dbg_sum) return go(wta_kernel<G, WIDE, 0, true>, G);           \
-        if (nplanes == 8) return go(wta_kernel<G, WIDE, 8, false>, G);     \
-        if (nplanes == 4) return go(wta_kernel<G, WIDE, 4, false>, G);     \
+#define SGM_WTA(G)                                                          \
+    case G:                                                                 \
+        if (dbg_sum) return go(wta_kernel<G, WIDE, 0, true>, G);            \
+        if (all && nplanes == 8) return go(wta_kernel<G, WIDE, 8, false>, G);\
+        if (all && nplanes == 4) return go(wta_kernel<G, WIDE, 4, false>, G);\
         return go(wta_kernel<G, WIDE, 0, false>, G)
     switch (256 / Dp) {  // pixels per warp
         SGM_WTA(32);
