@@ -241,15 +241,17 @@ int sgm_batch_device_bytes(sgm_batch b, size_t *bytes);
  * of 8: 1 (the default), 2 or 4, or SGM_AGG_CHUNKS_MIXED.  With 1 a lane holds
  * one chunk, or half of one on the long-axis scanlines (rows when W >= H) while
  * D <= 128, whose chain of steps sets the kernel's duration, and down to a
- * quarter of one on small images; with 2 and 4 it holds that many chunks in
+ * quarter of one on small images (D = 65 to 96 and 161 to 192 may take one and a
+ * half); with 2 and 4 it holds that many chunks in
  * every direction, and MIXED is one chunk on the long-axis scanlines and two
  * in the other directions (where D spans a power of two of chunks; else as 1).
  * SGM_ERR_UNSUPPORTED above what D allows (D must span at least that many
  * chunks; the 16-bit costs of SGM_COST_SAD take 1).  More disparities per lane
  * let a warp walk more scanlines at once with fewer instructions per
  * disparity estimate, but each step of a scanline takes longer.  Results do
- * not depend on either setting.  A new handle starts with 4 blocks per SM and
- * setting 1, or with what sgm_autotune chose for its shape. */
+ * not depend on either setting.  A new handle starts with setting 1 and 4 blocks
+ * per SM (5 for shapes whose work fills these better), or with what sgm_autotune
+ * chose for its shape. */
 #define SGM_AGG_CHUNKS_MIXED 3
 int sgm_set_aggregation(sgm_handle h, int blocks_per_sm, int chunks_per_lane);
 int sgm_get_aggregation(sgm_handle h, int *blocks_per_sm, int *chunks_per_lane);

@@ -2,14 +2,25 @@
 // volume (Eq. 1).
 //
 // Decomposition.  Every enabled direction cuts the image into independent
-// scanlines: rows for the horizontal directions, columns for the vertical
-// ones and W+H-1 diagonals for each diagonal direction.  The Dp disparities of
-// one pixel are held by LPS lanes, NP pairs of disparities per lane, so one
-// warp walks G = 32 / LPS neighbouring scanlines in lock-step.  The kernel is
-// persistent: blocks_per_sm blocks of 4 warps run on every SM and pull jobs
-// (one direction, G scanlines) from a work queue until it is empty.  Opposite
-// directions of the same scanlines are neighbouring jobs, so that the second
-// one finds the costs in L2.
+// scanlines.  Let W >= H (else swap the axes): rows for the horizontal
+// directions, and W scanlines of H steps, one row per step, for each of the six
+// others.  A diagonal that leaves the image on the left or right comes in again on
+// the other side of the next row, where its path starts anew, so all of them have
+// the same length.  The Dp disparities of one pixel are held by LPS lanes, NP pairs
+// of disparities per lane, so one warp walks G = 32 / LPS neighbouring scanlines in
+// lock-step.  The kernel is persistent: blocks_per_sm blocks of 4 warps run on
+// every SM and pull jobs (one direction, G scanlines) from a work queue until it is
+// empty.
+//
+// Sweeps.  The column and the two diagonals that go down start together, have the
+// same length and stay within a few rows of one another, so a row of costs is read
+// from HBM once for the three of them; the three that go up follow and start on the
+// rows that were read last.  1280 x 720, D = 192, 8 paths: 0.96 GB read where
+// directions one after the other read 1.18 GB (the costs are 0.18 GB), 1.37 GB
+// written.  Aggregation in us, directions one after the other -> sweeps: 1242 x 375,
+// D = 128, 8 paths 125 -> 116, 641 x 479, D = 97 90 -> 82, 480 x 752, D = 128 105
+// -> 97, 1920 x 1080, D = 192 1147 -> 1105 (with six pairs per lane), 1280 x 720,
+// D = 64 168 -> 154; 640 x 360, D = 60, three of the six directions, 32.8 -> 34.9.
 //
 // Arithmetic.  The record of a pixel is folded: pair k holds the disparities
 // (k, Dp-1-k), packed as two 16-bit halves, and a lane holds NP consecutive
@@ -23,15 +34,13 @@
 // lane).  One update is
 //     t = min(min(L(d-1), L(d+1), m + P2 - P1) + P1, L(d));   L' = t + C - m
 // (the same minimum as min(L(d±1) + P1, L(d), m + P2)): a three-way packed
-// minimum and a packed add-then-minimum.  8-bit path costs are kept without
-// the "- m" (U = L + the minima subtracted so far, brought back to zero every
-// half ring), so that the update ends in a two-input add; the bytes that are
-// stored are U - m.  16-bit path costs (SAD) leave no room for that and
-// subtract m at each step.  m = min_d L is reduced within the lane, folded over
-// the two halves, then reduced over the scanline's lanes: xor-shuffles
-// for scanlines of up to 4 lanes, one full-warp redux.sync per scanline of
-// the warp for wider ones.  Starting from L = 0, m = 0 makes the first step
-// produce L = C without a special case.
+// minimum, a packed add-then-minimum and a three-input add.  Keeping L without the
+// "- m" for some steps (a two-input add, m subtracted when storing) took fewer ALU
+// instructions and the same time (131-135 us against 128, 1242 x 375).  m = min_d L is
+// reduced within the lane, folded over the two halves, then reduced over the
+// scanline's lanes: xor-shuffles for scanlines of up to 4 lanes, one full-warp
+// redux.sync per scanline of the warp for wider ones.  Starting from L = 0, m = 0
+// makes the first step produce L = C without a special case.
 //
 // Padding.  Slots d >= D hold the cost 255 (0x7FFF for 16-bit costs).  As bits
 // + P2 <= 255 (cmax + P2 <= 0x7FFF), a padding slot's path cost is at least m +
@@ -52,12 +61,19 @@
 // by a 1 the compiler cannot see (the job table's unit field), which run on the
 // FMA pipe.
 //
-// Memory.  Costs are loaded one half ring (HB steps) ahead, all loads of a
-// half together: a warp has few scoreboards, so a wait for one load of a long
-// ring also waits for the youngest load that shares its scoreboard.  Each step
-// stores the lane's path costs to the direction's plane, in the cost volume's
-// order and width, with evict_first: the planes are read back only once, by
-// the WTA kernel.
+// Memory.  Costs come through a ring of four stages of 4 to 16 steps per warp in
+// shared memory, filled by 16-byte asynchronous copies: with loads into registers,
+// 16 steps ahead, a third of the warps' time was waits, as a warp has few
+// scoreboards and a wait for the oldest load also waited for the youngest (1242 x
+// 375, 8 paths: 149 -> 128 us).  Each step stores the lane's path costs to the
+// direction's plane, in the cost volume's order and width, with evict_first: the
+// planes are read back only once, by the WTA kernel (without it 125 -> 135 us).  The
+// planes of a sweep's directions are neighbours in a pixel's record (numbered by
+// direction instead: 900 x 901, D = 96, 254 us against 243).
+//
+// Bound.  At D = 128 and more it is HBM: 5.1 to 5.3 TB/s of reads and writes mixed, in
+// runs of a pixel's Dp bytes.  Small images are bound by the ALU pipe while all
+// scanlines run and by the long axis' chain of steps after that.
 
 #include <cuda_fp16.h>
 
@@ -72,17 +88,27 @@ namespace {
 constexpr int kSchedulers = 608;  // warp schedulers of the GPU (152 SMs)
 
 // Pairs per lane for a W x H image.  The base is 2 on the long axis and 4 in the
-// other directions (4 and 4 above D = 128).  Small images leave schedulers idle
-// and take as long as their longest chain of steps, so they get narrower lanes
-// (a step of one pair per lane and one scanline per warp takes 28 ns, of two and
-// two 40, of four and four 80; with D = 128, two and one 31, four and two 50).
-// Measured, aggregation in us:
-//   640 x 360, D = 60, 4 paths: base 37.6, (1, 4) 35.7, (1, 2) 32.8;  SAD 41.2, 38.6, 33.2
-//   640 x 480, D = 64, 4 paths: base 45.8, (1, 2) 39.1;  8 paths: base 69.4, (1, 2) 67.8, (2, 2) 61.3
-//   464 x 161, D = 64, 8 paths: base 28.8, (1, 4) 24.3, (1, 2) 28.0
-//   1280 x 720, D = 64, 8 paths: base 173.9, (1, 2) 176.4, (2, 2) 171.2
-//   320 x 240, D = 32, 4 paths: base 22.7, (1, 4) 22.8, (1, 1) 18.3;  1280 x 720, 8 paths: base 123.9, (1, 4) 132.9
-//   320 x 240, D = 128, 8 paths: base 35.0, (2, 2) 30.9;  480 x 752, 8 paths: base 102.8, (2, 2) 107.0
+// other directions (4 and 4 above D = 128).
+//
+// Small images leave schedulers idle and take as long as their longest chain of
+// steps, so they get narrower lanes (a step of one pair per lane and one scanline
+// per warp takes 28 ns, of two and two 40, of four and four 80; with D = 128, two
+// and one 31, four and two 50), as long as nearly all of their warps are resident at
+// once; where both sides of the image are alike the other directions' chain is the
+// longer one, and the long axis keeps 2.  Measured, aggregation in us:
+//   D = 64    640 x 360, 4 paths: base 40.7, (1, 4) 36.9, (1, 2) 34.8
+//             640 x 480, 4 paths: base 46.3, (1, 4) 54, (1, 2) 39.0, (2, 2) 38.6;  8 paths: 63.4, 71.7, 63.7, 56.1
+//             514 x 166, 8 paths: base 32.6, (1, 4) 26.8, (1, 2) 31.0;  437 x 1032: 83.3, 73.7, 91.4
+//             1280 x 720, 8 paths: base 154, (2, 2) 157
+//   D = 32    246 x 269, 8 paths: base 25.5, (1, 1) 18.7;  1280 x 720: base 123.9, (1, 4) 132.9
+//   D = 128   230 x 182, 8 paths: base 22.2, (2, 2) 19.5;  480 x 752: base 97.5, (2, 2) 104
+//
+// 96 and 192 slots are 12 or 24 lanes of four pairs, which leave a quarter of every
+// warp idle; 8 or 16 lanes of six fill it.  It pays where the diagonals read their
+// costs from L2 and the warps, fewer by a third, still fill the chip:
+//   D = 192   1920 x 1080, 8 paths: (4, 4) 1174, (4, 6) 1110;  570 x 280: 77, 72;  320 x 240: 42, 45
+//             1280 x 720, 4 paths: 248, 276
+//   D = 96    1784 x 799, 8 paths: (2, 4) 486, (2, 6) 460;  640 x 480: 86, 98
 LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool many) {
     const int Dp = padded_disparities(D);
     const bool pow2 = (Dp & (Dp - 1)) == 0;  // lanes of more than 4 pairs come in powers of two
@@ -90,8 +116,9 @@ LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool m
     if (!wide && pow2 && cpl == 4) return {16, 16};
     if (!wide && pow2 && cpl == kMixedCpl) return {4, 8};
     LaneConfig lc{Dp <= 128 ? 2 : 4, 4};
-    if (many || Dp < 32 || Dp > 128) return lc;
+    if (many || Dp < 32) return lc;
     const int axis = W >= H ? 0x03 : 0x0C;  // the long-axis directions
+    const int longer = W >= H ? W : H, shorter = W >= H ? H : W;
     long lines_long = 0, lines_other = 0;
     for (int r = 0; r < kMaxPaths; r++)
         if ((mask >> r) & 1) (((axis >> r) & 1) ? lines_long : lines_other) += scanlines_of(r, W, H);
@@ -103,10 +130,16 @@ LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool m
         if (warps(1, 4) <= 3 * kSchedulers) return {1, 4};
         return lc;
     }
-    // narrower lanes in the other directions where their chain is the longer one
-    const double chain_long = (Dp == 64 ? 28. : 31.) * (W >= H ? W : H), chain_other = (Dp == 64 ? 80. : 50.) * (W >= H ? H : W);
-    if (chain_other > chain_long && warps(2, 2) <= 12 * kSchedulers) lc.np_other = 2;
-    if (Dp == 64 && warps(1, lc.np_other) <= 3 * kSchedulers) lc.np_long = 1;
+    if (Dp == 64) {
+        // chain of the long axis at 2 pairs per lane against that of the others at 4
+        const bool square = 56. * longer < 80. * shorter, flat = 32. * longer > 80. * shorter;
+        if (warps(1, 2) <= (square ? 3. : 3.6) * kSchedulers && !flat) return {1, 2};
+        if (square) return warps(2, 2) <= 12 * kSchedulers ? LaneConfig{2, 2} : lc;
+        if (warps(1, 4) <= 4 * kSchedulers) return {1, 4};
+        return lc;
+    }
+    if (Dp <= 128 && 50. * shorter > 31. * longer && warps(2, 2) <= 4 * kSchedulers) lc.np_other = 2;
+    else if (!wide && Dp % 96 == 0 && (mask & 0xF0) && warps(lc.np_long, 6) >= 3 * kSchedulers) lc.np_other = 6;
     return lc;
 }
 
@@ -117,18 +150,19 @@ PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool 
     j.unit = 1u;
     const LaneConfig lc = lane_config(W, H, D, mask, wide, cpl, many);
     j.lanes = lc;
-    // long axis first, then the short axis, then the diagonals; each entry is a
-    // direction and its opposite
-    const int first[4] = {W >= H ? 0 : 2, W >= H ? 2 : 0, 4, 6};
-    for (int i = 0; i < 4; i++) {
+    const bool wide_image = W >= H;
+    auto along = [&](int r) { return wide_image ? dir_dy(r) : dir_dx(r); };  // step along the short axis
+    // entries: the long axis, all that moves along the short axis one way, and all that
+    // moves the other way
+    int planes = 0;
+    for (int i = 0; i < 3; i++) {
         const int k = j.n;
-        for (int o = 0; o < 2; o++) {
-            const int r = first[i] + o;
-            if (!((mask >> r) & 1)) continue;
+        for (int r = 0; r < kMaxPaths; r++) {
+            if (!((mask >> r) & 1) || along(r) != (i == 0 ? 0 : i == 1 ? 1 : -1)) continue;
             const int e = j.ndir[k]++;
             j.dx[k][e] = dir_dx(r);
             j.dy[k][e] = dir_dy(r);
-            j.plane[k][e] = __builtin_popcount((unsigned)mask & ((1u << r) - 1u));
+            j.plane[k][e] = planes++;
             j.nlines[k] = (int)scanlines_of(r, W, H);
         }
         if (j.ndir[k] == 0) continue;
@@ -138,6 +172,20 @@ PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool 
         if (i == 0) j.nlong = j.jbegin[k + 1];
     }
     return j;
+}
+
+// 16 resident warps per SM, or 20 where these leave the last round of short-axis
+// jobs less than half full and 20 do not (the long-axis jobs outlast several rounds).
+// Measured, aggregation in us at 4 and 5 blocks per SM, 8 paths:
+//   rounds of 2.2 and 1.6 (1242 x 375, D = 128) 127, 116;  2.4 and 1.6 (1000 x 600, D = 128) 161, 155
+//   1.5 and 0.9 (656 x 572, D = 128) 104, 114;  2.6 and 1.9 (1400 x 400, D = 128) 139, 148
+//   1.1 and 0.8 (1280 x 720, D = 64) 155, 172;  2.1 and 1.5 (1920 x 1080, D = 64) 381, 393
+int default_blocks_per_sm(const PathJobs &j) {
+    const double others = j.jbegin[j.n] - j.nlong;
+    auto rounds = [&](int blocks) { return others / (blocks * kSchedulers - j.nlong); };
+    if (4 * kSchedulers <= j.nlong) return 4;
+    const double r4 = rounds(4), r5 = rounds(5);
+    return r5 > 1 && r4 - (int)r4 < 0.5 && r5 - (int)r5 > 0.5 ? 5 : 4;
 }
 
 namespace {
@@ -196,7 +244,8 @@ struct Blk {
     static constexpr bool kHalf = NP == 1 && !WIDE;
     static constexpr int kLane = WIDE ? 4 * NP : 2 * NP;  // bytes of a lane
     static constexpr int kWords = WIDE ? NP : NP == 1 ? 1 : NP / 2;
-    static_assert(kWords == 1 || kWords == 2 || kWords % 4 == 0, "a lane block is 4, 8 or whole 16-byte vectors");
+    static constexpr bool kStaged = kWords == 3;  // no vector: stored by way of shared memory
+    static_assert(kWords <= 3 || kWords % 4 == 0, "a lane block is 4, 8, 12 or whole 16-byte vectors");
     uint32_t w[kWords];
 };
 
@@ -207,6 +256,9 @@ __device__ __forceinline__ Blk<NP, WIDE> ld_ring(uint32_t at) {
         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v.w[0]) : "r"(at));
     } else if constexpr (Blk<NP, WIDE>::kWords == 2) {
         asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.w[0]), "=r"(v.w[1]) : "r"(at));
+    } else if constexpr (Blk<NP, WIDE>::kStaged) {
+#pragma unroll
+        for (int q = 0; q < 3; q++) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v.w[q]) : "r"(at + 4 * q));
     } else {
 #pragma unroll
         for (int q = 0; q < Blk<NP, WIDE>::kWords; q += 4)
@@ -235,6 +287,15 @@ __device__ __forceinline__ void st_blk(Blk<NP, WIDE> *p, const Blk<NP, WIDE> &v,
     }
 }
 
+// Stores 16 bytes of a step that the lanes have left in shared memory at `from`.
+__device__ __forceinline__ void st_staged(uint4 *p, uint32_t from, uint64_t pol) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(from) : "memory");
+    asm volatile("st.global.L1::no_allocate.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
+                 : "memory");
+}
+
 // The cost ring of a warp: kStages stages of one block of steps each, in shared
 // memory.  A step is the warp's 32 lane blocks; one asynchronous copy of the
 // warp moves kCopy bytes per lane, kPer steps together (or a part of one).
@@ -245,9 +306,11 @@ struct Ring {
     static constexpr int kCopy = kTiny ? 8 : 16;
     static constexpr int kPer = 32 * kCopy >= kStep ? 32 * kCopy / kStep : 1;     // steps of a copy
     static constexpr int kParts = 32 * kCopy >= kStep ? 1 : kStep / (32 * kCopy);  // copies of a step
-    static constexpr int kBlock = kRingBytes / kStages / kStep < 16 ? kRingBytes / kStages / kStep : 16;  // steps of a stage
+    static constexpr int kFit = kRingBytes / kStages / kStep;
+    static constexpr int kBlock = kFit >= 16 ? 16 : kFit > 4 ? kFit & ~3 : kFit;  // steps of a stage
     static constexpr int kBytes = kBlock * kStep;
-    static_assert(kStages * kBytes <= kRingBytes, "the ring holds the stages");
+    static constexpr int kStageOut = Blk<NP, WIDE>::kStaged ? 2 * kStep : 0;  // path costs on their way out, behind the stages
+    static_assert(kStages * kBytes + kStageOut <= kRingBytes, "the ring holds the stages");
 };
 
 // Asynchronous copies of BYTES into shared memory (zeros when ok is false).
@@ -387,41 +450,33 @@ __device__ __forceinline__ Blk<NP, WIDE> path_step(PathState<NP> &st, const Blk<
     return out;
 }
 
-// First pixel and length of scanline s of direction (dx, dy).  A direction and
-// its opposite number their scanlines alike (rows, columns, x - y or x + y).
-__device__ __forceinline__ void line_start(int dx, int dy, int s, int W, int H, int &x, int &y, int &len) {
-    if (dy == 0) {
-        y = s;
-        x = dx > 0 ? 0 : W - 1;
-        len = W;
-    } else if (dx == 0) {
-        x = s;
-        y = dy > 0 ? 0 : H - 1;
-        len = H;
-    } else if (dx == dy) {
-        x = max(s - (H - 1), 0);
-        y = max((H - 1) - s, 0);
-        len = min(W - x, H - y);
-        if (dy < 0) {
-            x += len - 1;
-            y += len - 1;
-        }
-    } else {
-        x = min(s, W - 1);
-        y = s - x;
-        len = min(x + 1, H - y);
-        if (dy < 0) {
-            x -= len - 1;
-            y += len - 1;
-        }
+// Scanline s of direction (dx, dy): its first pixel, the step before which it
+// wraps (kNever: never) and what the wrap adds to the pixel index.
+constexpr int kNever = 0x3FFFFFFF;
+struct Walk {
+    int x, y, wrap, jump;
+};
+__device__ __forceinline__ Walk walk_of(int dx, int dy, int s, int W, int H) {
+    const bool by_rows = dx == 0 || (dy != 0 && W >= H);  // one row per step, from column s
+    Walk w;
+    w.x = by_rows ? s : dx > 0 ? 0 : W - 1;
+    w.y = by_rows ? dy > 0 ? 0 : H - 1 : s;
+    w.wrap = kNever;
+    w.jump = 0;
+    if (dx != 0 && dy != 0) {
+        const int n = by_rows ? W : H, step = by_rows ? dx : dy;
+        w.wrap = step > 0 ? n - s : s + 1;
+        w.jump = -step * (by_rows ? W : H * W);
     }
+    return w;
 }
 
 // One job: the G neighbouring scanlines s0 .. s0+G-1 of one direction
 // (dx, dy), scanline s0 + grp for this lane's group, written to plane
 // `plane` of `nplanes`.  A scanline's pixel is LPS lane blocks of NP pairs.
 // FULL: the G scanlines' lanes fill the warp.
-template <int NP, int G, bool WIDE, bool FULL>
+// WRAP: diagonals may be among the directions.
+template <int NP, int G, bool WIDE, bool FULL, bool WRAP>
 __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__restrict__ planes_, int W, int H,
                                         int lps_, int nplanes, int dx, int dy, int plane, int nlines, int s0,
                                         uint32_t P1x2, uint32_t P2x2, uint64_t pol, uint32_t one) {
@@ -444,43 +499,70 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     lg.lo_mark = lg.first ? 0x7FFF7FFFu : 0u;
     lg.sel_c = lg.li & 1 ? 0x4240u : 0x4341u;
     // Likewise scanlines beyond the last repeat it.
-    int x, y, len;
-    line_start(dx, dy, min(s0 + lg.grp, nlines - 1), W, H, x, y, len);
-    const int steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
-    const int minlen = (int)__reduce_min_sync(0xffffffffu, (unsigned)len);
+    const Walk wk = walk_of(dx, dy, min(s0 + lg.grp, nlines - 1), W, H);
+    const int len = dx == 0 || (dy != 0 && W >= H) ? H : W;
     // block indices: cost block (x, y, li) is cost[(y*W + x)*LPS + li], plane
     // block is planes[((y*W + x)*nplanes + plane)*LPS + li] (all planes of a
     // pixel are adjacent).  They stay below 2^32 (checked at handle creation).
-    const long long pix = (long long)y * W + x, dir = (long long)dy * W + dx;
+    const long long pix = (long long)wk.y * W + wk.x, dir = (long long)dy * W + dx;
     const int rec = LPS * BT::kLane;  // bytes of a pixel's record
     const long long cost_copies = (long long)W * H * rec / RT::kCopy;
-    const long long plane_blocks = (long long)W * H * nplanes * rec / (int)sizeof(BT);
+    const long long plane_blocks = (long long)W * H * nplanes * rec / (BT::kStaged ? 16 : (int)sizeof(BT));
     // the lane block of the step to store (their count stays below 2^32, checked at
     // handle creation; 32 bits keep the address arithmetic on the FMA pipe)
-    uint32_t oi = (uint32_t)(((pix * nplanes + plane) * rec + lg.li * BT::kLane) / (int)sizeof(BT));
-    const uint32_t ostep = (uint32_t)(dir * nplanes * rec / (int)sizeof(BT));
-    const bool stores = !BT::kHalf || !(lg.li & 1);
+    constexpr int kUnit = BT::kStaged ? 16 : (int)sizeof(BT);  // bytes of a store
+    uint32_t oi = (uint32_t)(((pix * nplanes + plane) * rec + lg.li * BT::kLane) / kUnit);
+    const uint32_t ostep = (uint32_t)(dir * nplanes * rec / kUnit);
+    const uint32_t ojump = (uint32_t)((long long)wk.jump * nplanes * rec / kUnit);
+    bool stores = !BT::kHalf || !(lg.li & 1);
+    int owrap = wk.wrap;  // of the scanline this lane stores for
+    if constexpr (BT::kStaged) {
+        const int ogrp = lane * 16 / rec;
+        const Walk ow = walk_of(dx, dy, min(s0 + ogrp, nlines - 1), W, H);
+        stores = ogrp < G;
+        owrap = ow.wrap;
+        oi = (uint32_t)(((((long long)ow.y * W + ow.x) * nplanes + plane) * rec + lane * 16 - ogrp * rec) / 16);
+    }
     // this lane's share of the copies: kCopy bytes at offset ccol of the record of
     // scanline s0 + cgrp (one per part of a step), csub steps into the copy
     const int csub = lane * RT::kCopy / RT::kStep;
-    int clen[RT::kParts];
+    int cwrap[RT::kParts];
     bool mine[RT::kParts];  // a step's records may be shorter than the warp's copies
     uint32_t ci[RT::kParts];  // in units of kCopy bytes, below 2^32 like oi
 #pragma unroll
     for (int p = 0; p < RT::kParts; p++) {
         const int unit = (p * 32 + lane) * RT::kCopy % RT::kStep;  // byte of the step
         const int cgrp = unit / rec;
-        int cx, cy;
-        line_start(dx, dy, min(s0 + cgrp, nlines - 1), W, H, cx, cy, clen[p]);
-        mine[p] = FULL || cgrp < G;
-        ci[p] = (uint32_t)((((long long)cy * W + cx + csub * dir) * rec + (unit - cgrp * rec)) / RT::kCopy);
+        const Walk cw = walk_of(dx, dy, min(s0 + cgrp, nlines - 1), W, H);
+        cwrap[p] = cw.wrap;
+        mine[p] = BT::kStaged ? lane * RT::kCopy < RT::kStep : FULL || cgrp < G;
+        ci[p] = (uint32_t)((((long long)cw.y * W + cw.x + csub * dir) * rec + (unit - cgrp * rec)) / RT::kCopy);
     }
+    const uint32_t cjump = (uint32_t)((long long)wk.jump * rec / RT::kCopy);
     const uint32_t cadv = (uint32_t)(dir * RT::kPer * rec / RT::kCopy);
     const uint32_t ring_w = ring + lane * RT::kCopy, ring_r = ring + (vl * BT::kLane & ~3);
     using CT = typename std::conditional<RT::kCopy == 16, uint4, uint2>::type;
     const CT *__restrict__ cost = reinterpret_cast<const CT *>(cost_);
     BT *__restrict__ planes = reinterpret_cast<BT *>(planes_);
+    const uint32_t out = ring + kStages * RT::kBytes;  // [2][kStep], BT::kStaged only
+    // Stores the path costs of step i of a block, where ok.
+    auto put = [&](int i, const BT &o, bool ok) {
+        if constexpr (BT::kStaged) {
+            // two buffers: a lane writes one again only after the barrier of the step
+            // between, which follows every lane's read of it
+            const uint32_t buf = out + (uint32_t)(i & 1) * RT::kStep;
+#pragma unroll
+            for (int q = 0; q < 3; q++)
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(buf + lane * BT::kLane + 4 * q), "r"(o.w[q]) : "memory");
+            __syncwarp();
+            if (ok && in_range(oi, plane_blocks)) st_staged(reinterpret_cast<uint4 *>(planes_) + oi, buf + lane * 16, pol);
+        } else {
+            if (ok && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
+        }
+        oi += ostep;
+    };
     // Copies block `blk` into its stage; what a scanline does not have reads as 0.
+    // checked: the block may be past the end or hold a wrap.
     auto fetch = [&](int blk, auto checked) {
         const uint32_t at = ring_w + (uint32_t)(blk % kStages) * RT::kBytes;
 #pragma unroll
@@ -489,13 +571,28 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
             for (int p = 0; p < RT::kParts; p++) {
                 const uint32_t to = at + i * RT::kStep + p * 32 * RT::kCopy;
                 if constexpr (decltype(checked)::value) {
-                    const bool ok = mine[p] && blk * RT::kBlock + i + csub < clen[p] && in_range(ci[p], cost_copies);
-                    copy_or_zero<RT::kCopy>(to, cost + (ok ? ci[p] : 0u), ok);
+                    const int t = blk * RT::kBlock + i + csub;
+                    if (WRAP && t >= cwrap[p]) {
+                        ci[p] += cjump;
+                        cwrap[p] = kNever;
+                    }
+                    const bool ok = mine[p] && t < len && in_range(ci[p], cost_copies);
+                    if (!BT::kStaged || mine[p]) copy_or_zero<RT::kCopy>(to, cost + (ok ? ci[p] : 0u), ok);
                 } else if (mine[p] && in_range(ci[p], cost_copies)) {
                     copy_async<RT::kCopy>(to, cost + ci[p]);
                 }
                 ci[p] += cadv;
             }
+        }
+        if constexpr (WRAP && decltype(checked)::value) {
+            // a lane that copies every kPer-th step may have its first one past the
+            // wrap in the next block
+#pragma unroll
+            for (int p = 0; p < RT::kParts; p++)
+                if (cwrap[p] < (blk + 1) * RT::kBlock) {
+                    ci[p] += cjump;
+                    cwrap[p] = kNever;
+                }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -511,50 +608,72 @@ __device__ __forceinline__ void run_job(const void *__restrict__ cost_, void *__
     __syncwarp();  // the ring of the warp's previous job has been read
 #pragma unroll 1
     for (int j = 0; j < kStages - 1; j++) fetch(j, Checked());
-    int blk = 0;
-    // While every scanline of the warp has all the steps of the block, stores need
-    // no checks, nor do the copies while it has those of the block being fetched.
-#pragma unroll 1
-    for (; (blk + 1) * B <= minlen; blk++) {
+    // Blocks of steps: nblk, the first nfull of them whole; [wrap0, wrap1) may hold a wrap.
+    const int nblk = (len + B - 1) / B, nfull = len / B;
+    const int wrap0 = WRAP ? min((int)__reduce_min_sync(0xffffffffu, (unsigned)wk.wrap) / B, nblk) : nblk;
+    const int wrap1 = WRAP ? min((int)__reduce_max_sync(0xffffffffu, (unsigned)wk.wrap) / B + 1, nblk) : nblk;
+    auto next_block = [&](int blk) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
         __syncwarp();  // every lane's copies of this block are there, and the block before has been read
-        if ((blk + kStages) * B <= minlen) fetch(blk + kStages - 1, Unchecked());
-        else fetch(blk + kStages - 1, Checked());
-        const uint32_t at = ring_r + (uint32_t)(blk % kStages) * RT::kBytes;
+        const int ahead = blk + kStages - 1;
+        if (ahead < nfull && (ahead < wrap0 || ahead >= wrap1)) fetch(ahead, Unchecked());
+        else fetch(ahead, Checked());
+        return ring_r + (uint32_t)(blk % kStages) * RT::kBytes;
+    };
+    constexpr int kTail = B < 4 ? B : 4;
+    static_assert(B % kTail == 0, "whole parts of a block");
+    // a block in which nothing ends or wraps: no checks
+    auto plain = [&](int blk) {
+        const uint32_t at = next_block(blk);
         BT cur = ld_ring<NP, WIDE>(at);
 #pragma unroll
         for (int i = 0; i < B; i++) {
             BT nxt = cur;
             if (i + 1 < B) nxt = ld_ring<NP, WIDE>(at + (i + 1) * RT::kStep);
             const BT o = path_step<NP, G, WIDE>(st, cur, P1x2, QPx2, lg, one);
-            if (stores && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
-            oi += ostep;
+            put(i, o, stores);
             cur = nxt;
         }
-    }
-    // The blocks in which some scanline ends, a few steps at a time: what a
-    // scanline computes past its end is not stored.
-    constexpr int kTail = B < 4 ? B : 4;
-    static_assert(B % kTail == 0, "whole parts of a block");
+    };
+    // any other, a few steps at a time: what is computed past the end is not stored
+    auto special = [&](int blk) {
+        const uint32_t at = next_block(blk);
 #pragma unroll 1
-    for (; blk * B < steps; blk++) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
-        __syncwarp();
-        fetch(blk + kStages - 1, Checked());
-        const uint32_t at = ring_r + (uint32_t)(blk % kStages) * RT::kBytes;
-#pragma unroll 1
-        for (int i = 0; i < B && blk * B + i < steps; i += kTail) {
-            const int left = len - blk * B - i;
+        for (int i = 0; i < B && blk * B + i < len; i += kTail) {
             BT in[kTail];
 #pragma unroll
             for (int q = 0; q < kTail; q++) in[q] = ld_ring<NP, WIDE>(at + (i + q) * RT::kStep);
 #pragma unroll
             for (int q = 0; q < kTail; q++) {
+                const int t = blk * B + i + q;
+                if (WRAP && t == wk.wrap) {
+#pragma unroll
+                    for (int k = 0; k < NP; k++) st.R[k] = 0u;
+                    st.m2 = 0u;
+                    st.mQ = QPx2;
+                }
+                if (WRAP && t == owrap) oi += ojump;
                 const BT o = path_step<NP, G, WIDE>(st, in[q], P1x2, QPx2, lg, one);
-                if (stores && q < left && in_range(oi, plane_blocks)) st_blk(planes + oi, o, pol);
-                oi += ostep;
+                put(q, o, stores && t < len);
             }
         }
+    };
+    int blk = 0;
+    if constexpr (WRAP) {
+        const int cut = min(wrap0, nfull);
+#pragma unroll 1
+        for (; blk < cut; blk++) plain(blk);
+#pragma unroll 1
+        for (; blk < wrap1; blk++) special(blk);
+#pragma unroll 1
+        for (; blk < nfull; blk++) plain(blk);
+#pragma unroll 1
+        for (; blk < nblk; blk++) special(blk);
+    } else {
+#pragma unroll 1
+        for (; blk < nfull; blk++) plain(blk);
+#pragma unroll 1
+        for (; blk < nblk; blk++) special(blk);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
@@ -575,12 +694,12 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
         int k = 0;
         while (job >= jobs.jbegin[k + 1]) k++;
         const int q = job - jobs.jbegin[k];
-        const int e = jobs.ndir[k] == 2 ? q & 1 : 0, line = jobs.ndir[k] == 2 ? q >> 1 : q;
+        const int line = q / jobs.ndir[k], e = q - line * jobs.ndir[k];
         if (job < jobs.nlong)
-            run_job<NPL, GL, WIDE, FULL>(cost, planes, W, H, Dp / (2 * NPL), nplanes, jobs.dx[k][e], jobs.dy[k][e],
+            run_job<NPL, GL, WIDE, FULL, false>(cost, planes, W, H, Dp / (2 * NPL), nplanes, jobs.dx[k][e], jobs.dy[k][e],
                                    jobs.plane[k][e], jobs.nlines[k], line * GL, P1x2, P2x2, pol, jobs.unit);
         else
-            run_job<NPO, GO, WIDE, FULL>(cost, planes, W, H, Dp / (2 * NPO), nplanes, jobs.dx[k][e], jobs.dy[k][e],
+            run_job<NPO, GO, WIDE, FULL || NPO == 6, true>(cost, planes, W, H, Dp / (2 * NPO), nplanes, jobs.dx[k][e], jobs.dy[k][e],
                                    jobs.plane[k][e], jobs.nlines[k], line * GO, P1x2, P2x2, pol, jobs.unit);
         job = next_job(job_counter, total, lane);
     }
@@ -624,10 +743,10 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
         int k = 0;
         while (local >= p.jobs.jbegin[k + 1]) k++;
         const int ql = local - p.jobs.jbegin[k];
-        const int e = p.jobs.ndir[k] == 2 ? ql & 1 : 0, line = p.jobs.ndir[k] == 2 ? ql >> 1 : ql;
+        const int line = ql / p.jobs.ndir[k], e = ql - line * p.jobs.ndir[k];
         auto job_as = [&](auto np, auto g) {
             constexpr int NP = decltype(np)::value, G = decltype(g)::value;
-            run_job<NP, G, WIDE, (G >= 8)>(p.cost, p.planes, p.W, p.H, p.Dp / (2 * NP), p.nplanes, p.jobs.dx[k][e],
+            run_job<NP, G, WIDE, (G >= 8), true>(p.cost, p.planes, p.W, p.H, p.Dp / (2 * NP), p.nplanes, p.jobs.dx[k][e],
                                  p.jobs.dy[k][e], p.jobs.plane[k][e], p.jobs.nlines[k], line * G, P1x2, P2x2, pol,
                                  p.jobs.unit);
         };
@@ -685,7 +804,10 @@ AggKernel agg_kernel_t(int Dp, LaneConfig lc) {
     SGM_AGG(2, 1, 2, 1);
     SGM_AGG_F(4, 1, 4, 1, false);  // 160, 192, 224
     SGM_AGG(4, 1, 4, 1);    // 256
-    if constexpr (!WIDE) {  // Dp a power of two, 16 to 256
+    if constexpr (!WIDE) {
+        SGM_AGG_F(2, 1, 6, 4, false);  // 96
+        SGM_AGG_F(4, 1, 6, 2, false);  // 192
+        // Dp a power of two, 16 to 256
         SGM_AGG(8, 32, 8, 32);
         SGM_AGG(8, 16, 8, 16);
         SGM_AGG(8, 8, 8, 8);
@@ -746,7 +868,7 @@ cudaError_t launch_aggregate(const uint8_t *cost, int W, int H, int D, int P1, i
     if (e != cudaSuccess) return e;
     // no more blocks than the jobs fill
     const int wanted = sms * (blocks_per_sm > 0 ? blocks_per_sm : 2), filled = (jobs.jbegin[jobs.n] + kWarps - 1) / kWarps;
-    const int blocks = filled < sms ? sms : filled < wanted ? filled : wanted;
+    const int blocks = filled < sms ? sms : filled < wanted ? filled : wanted;  // whole layers
     const int Dp = padded_disparities(D);
     const LaneConfig lc = jobs.lanes;
     const uint32_t P1x2 = (uint32_t)P1 * 0x00010001u, P2x2 = (uint32_t)P2 * 0x00010001u;

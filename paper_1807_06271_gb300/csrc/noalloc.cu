@@ -167,7 +167,7 @@ extern "C" int sgm_compute_static(int W, int H, int D, const sgm_params *params,
     }
     if (e == cudaSuccess)
         e = sgm::launch_aggregate(cost, W, H, D, params->P1, params->P2, wide, jobs, planes, npaths,
-                                  counter, 2, cpl, s);
+                                  counter, sgm::default_blocks_per_sm(jobs), cpl, s);
     if (e == cudaSuccess)
         e = sgm::launch_wta(planes, npaths, W, H, D, wide, params->lr_tolerance, disp_lr, nullptr, nullptr,
                             nullptr, s);

@@ -338,13 +338,10 @@ int sgm_create(int W, int H, int D, const sgm_params *params, sgm_handle *out) {
         cudaGetLastError();
         return SGM_ERR_CUDA;
     }
-    for (int r = 0; r < kMaxPaths; r++)
-        if ((params->path_mask >> r) & 1) h->path_of_plane[h->npaths++] = r;
+    h->npaths = __builtin_popcount((unsigned)params->path_mask);
     h->Dp = padded_disparities(D);
-    // 16 resident warps per SM (1242 x 375, D = 128, 8 paths: 128 us, against 133 with
-    // 12, 145 with 8 and 127 with 20); small images fill fewer
-    h->agg_blocks_per_sm = 4;
-    h->agg_cpl = 1;  // fastest for single pairs on every measured shape but portraits
+    h->agg_cpl = 1;  // fastest for single pairs on every measured shape
+    h->agg_blocks_per_sm = default_blocks_per_sm(make_path_jobs(W, H, D, params->path_mask, h->wide != 0, h->agg_cpl));
     h->schedule = SGM_SCHEDULE_PLANES;
     h->sweep_rows = 4;
     const Tuning tuned = tuned_for(h);

@@ -44,7 +44,6 @@ struct sgm_handle_s {
     int wide;        // 1: 16-bit costs and path costs (SAD), 0: 8-bit (census)
     int device;
     int npaths;
-    int path_of_plane[sgm::kMaxPaths];
 
     int Dp;          // padded disparities per pixel (8 * lanes per scanline)
 

@@ -21,12 +21,14 @@ __host__ __device__ constexpr int dir_dy(int r) {
     return r == 0 ? 0 : r == 1 ? 0 : r == 2 ? 1 : r == 3 ? -1 : r == 4 ? 1 : r == 5 ? -1 : r == 6 ? 1 : -1;
 }
 
-// Number of scanlines of direction r in a W x H image.
+// Number of scanlines of direction r in a W x H image.  Diagonals move along the
+// short axis and wrap around the long one (where the path starts anew), so that
+// all of them have the length of the short axis.
 inline long scanlines_of(int r, int W, int H) {
-    int dx = dir_dx(r), dy = dir_dy(r);
+    const int dx = dir_dx(r), dy = dir_dy(r);
     if (dy == 0) return H;
     if (dx == 0) return W;
-    return (long)W + H - 1;
+    return W >= H ? W : H;
 }
 
 // Rectification maps of the left and right image (device, W x H each; all
@@ -140,8 +142,6 @@ __host__ __device__ constexpr int fold_slot(int d, int Dp, bool wide) {
 // Cost of the padding slots.  With it they never hold a scanline's minimum nor
 // help a neighbour (census bits + P2 <= 255; SAD cmax + P2 < 0x7FFF).
 constexpr unsigned kPadCost = 255u, kPadCostWide = 0x7FFFu;
-// Planes one after the other, or all planes of a pixel back to back.
-constexpr bool kPlanar = false;
 
 // Pairs of disparities a lane of the aggregation kernel holds, for the
 // long-axis scanlines and for the other directions.
@@ -150,19 +150,20 @@ struct LaneConfig {
 };
 inline int lanes_of(int D, int np) { return padded_disparities(D) / (2 * np); }
 
-// Work list of the aggregation kernel: entry k is one enabled direction, or a
-// direction and its opposite, whose nlines scanlines are cut into jobs of G
+// Work list of the aggregation kernel: entry k is a set of enabled directions (the
+// two of the long axis, then the up to three that move along the short axis one
+// way and those that move the other way) whose nlines scanlines are cut into jobs of G
 // neighbouring scanlines (one warp each, G = 32 / lanes per scanline); the jobs
-// of the two directions alternate.  Job j belongs to entry k when jbegin[k] <=
-// j < jbegin[k+1].
+// of the directions alternate.  Job j belongs to entry k when jbegin[k] <= j <
+// jbegin[k+1].
 struct PathJobs {
     LaneConfig lanes;
     int n;                       // number of entries
-    int ndir[kMaxPaths / 2];     // directions of entry k
-    int dx[kMaxPaths / 2][2], dy[kMaxPaths / 2][2];
-    int plane[kMaxPaths / 2][2];  // their output planes
-    int nlines[kMaxPaths / 2];
-    int jbegin[kMaxPaths / 2 + 1];
+    int ndir[3];               // directions of entry k
+    int dx[3][3], dy[3][3];
+    int plane[3][3];           // their output planes, numbered in this order
+    int nlines[3];
+    int jbegin[4];
     int nlong;                   // jobs [0, nlong) belong to the long-axis directions
     uint32_t unit;               // always 1; see the kernel's multiply-adds
 };
@@ -171,11 +172,12 @@ struct PathJobs {
 // beyond the warps' first ones (cleared before every launch).
 constexpr size_t kJobStateBytes = 4224;
 
-// Builds the work list for the directions in `mask` (planes numbered in
-// increasing direction order), longest scanlines first, under the
+// Builds the work list for the directions in `mask`, longest scanlines first, under the
 // sgm_set_aggregation setting cpl.  many: other pairs' work runs beside it, so
 // the lanes are not narrowed to shorten a small image's chains.
 PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool many = false);
+// Resident 4-warp blocks per SM for a handle whose caller sets none.
+int default_blocks_per_sm(const PathJobs &jobs);
 // The most chunks per lane the aggregation takes for D (1 for 16-bit costs, up to 4).
 int chunks_per_lane_max(int D, bool wide);
 // Chunks-per-lane code of the mixed layout: long-axis scanlines at 1, the others at 2.
