@@ -494,10 +494,9 @@ def kernel_rooflines(w, stage, peaks, hbm_gbs):
     stage pass's mean event times."""
     de = w.de_per_frame
     npaths = bin(w.path_mask).count("1")
-    lanes = 1
-    while 8 * lanes < w.D:
-        lanes *= 2
-    Dp, eb = 8 * lanes, (2 if w.cost == 1 else 1)
+    # slots per pixel: 8, 16 or the multiple of 32 that holds D
+    Dp = 8 if w.D <= 8 else 16 if w.D <= 16 else (w.D + 31) // 32 * 32
+    eb = 2 if w.cost == 1 else 1
     out = {}
 
     def mean_s(k):

@@ -45,7 +45,7 @@ struct sgm_handle_s {
     int device;
     int npaths;
 
-    int Dp;          // padded disparities per pixel (8 * lanes per scanline)
+    int Dp;          // slots per pixel (padded_disparities)
 
     // every device allocation of the handle (scratch and staging), freed by sgm_destroy
     sgm::DevAlloc allocs[sgm::kMaxAllocs];
