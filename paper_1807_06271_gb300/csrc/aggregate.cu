@@ -20,7 +20,7 @@
 // written.  Aggregation in us, directions one after the other -> sweeps: 1242 x 375,
 // D = 128, 8 paths 125 -> 116, 641 x 479, D = 97 90 -> 82, 480 x 752, D = 128 105
 // -> 97, 1920 x 1080, D = 192 1147 -> 1105 (with six pairs per lane), 1280 x 720,
-// D = 64 168 -> 154; 640 x 360, D = 60, three of the six directions, 32.8 -> 34.9.
+// D = 64 168 -> 154 (and with the rows between the sweeps 1053 for 1920 x 1080); 640 x 360, D = 60, three of the six directions, 32.8 -> 34.9.
 //
 // Arithmetic.  The record of a pixel is folded: pair k holds the disparities
 // (k, Dp-1-k), packed as two 16-bit halves, and a lane holds NP consecutive
@@ -155,7 +155,17 @@ PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool 
     // entries: the long axis, all that moves along the short axis one way, and all that
     // moves the other way
     int planes = 0;
-    for (int i = 0; i < 3; i++) {
+    // Their order: the long axis first, as its chains are the longest, unless the costs
+    // are more than L2 keeps.  Then they come between the sweeps, whose warps must all
+    // run at once to share them.  Measured, long axis first and second, us (8 paths): 1920
+    // x 1080, D = 192 (398 MB) 1102, 1053;  1280 x 720, D = 192 (177 MB) 462, 425;  1920 x
+    // 1080, D = 64 (133 MB) 386, 365;  1280 x 720, D = 128 (118 MB) 264, 258;  1500 x 500, D
+    // = 128 (96 MB) 204, 210;  1242 x 375, D = 192 (89 MB) 196, 199;  900 x 700, D = 96 (60
+    // MB) 157, 188.  1280 x 720, D = 128, 4 paths without diagonals: 152, 155.
+    const double volume = (double)W * H * padded_disparities(D) * (wide ? 2 : 1);
+    const bool sweeps_first = !many && volume >= 100e6 && (mask & 0xF0);
+    j.klong = -1;
+    for (int i : {sweeps_first ? 1 : 0, sweeps_first ? 0 : 1, 2}) {
         const int k = j.n;
         for (int r = 0; r < kMaxPaths; r++) {
             if (!((mask >> r) & 1) || along(r) != (i == 0 ? 0 : i == 1 ? 1 : -1)) continue;
@@ -169,7 +179,7 @@ PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool 
         const int G = 32 / lanes_of(D, i == 0 ? lc.np_long : lc.np_other);
         j.jbegin[k + 1] = j.jbegin[k] + j.ndir[k] * ((j.nlines[k] + G - 1) / G);
         j.n++;
-        if (i == 0) j.nlong = j.jbegin[k + 1];
+        if (i == 0) j.nlong = j.jbegin[k + 1] - j.jbegin[k], j.klong = k;
     }
     return j;
 }
@@ -183,7 +193,7 @@ PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool 
 int default_blocks_per_sm(const PathJobs &j) {
     const double others = j.jbegin[j.n] - j.nlong;
     auto rounds = [&](int blocks) { return others / (blocks * kSchedulers - j.nlong); };
-    if (4 * kSchedulers <= j.nlong) return 4;
+    if (j.klong != 0 || 4 * kSchedulers <= j.nlong) return 4;
     const double r4 = rounds(4), r5 = rounds(5);
     return r5 > 1 && r4 - (int)r4 < 0.5 && r5 - (int)r5 > 0.5 ? 5 : 4;
 }
@@ -695,7 +705,7 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
         while (job >= jobs.jbegin[k + 1]) k++;
         const int q = job - jobs.jbegin[k];
         const int line = q / jobs.ndir[k], e = q - line * jobs.ndir[k];
-        if (job < jobs.nlong)
+        if (k == jobs.klong)
             run_job<NPL, GL, WIDE, FULL, false>(cost, planes, W, H, Dp / (2 * NPL), nplanes, jobs.dx[k][e], jobs.dy[k][e],
                                    jobs.plane[k][e], jobs.nlines[k], line * GL, P1x2, P2x2, pol, jobs.unit);
         else

@@ -152,29 +152,31 @@ inline int lanes_of(int D, int np) { return padded_disparities(D) / (2 * np); }
 
 // Work list of the aggregation kernel: entry k is a set of enabled directions (the
 // two of the long axis, then the up to three that move along the short axis one
-// way and those that move the other way) whose nlines scanlines are cut into jobs of G
-// neighbouring scanlines (one warp each, G = 32 / lanes per scanline); the jobs
-// of the directions alternate.  Job j belongs to entry k when jbegin[k] <= j <
-// jbegin[k+1].
+// way and those that move the other way; large images take the long axis second)
+// whose nlines scanlines are cut into jobs of G neighbouring scanlines (one warp
+// each, G = 32 / lanes per scanline); the jobs of the directions alternate.  Job j
+// belongs to entry k when jbegin[k] <= j < jbegin[k+1].
 struct PathJobs {
     LaneConfig lanes;
-    int n;                       // number of entries
+    int n;                     // number of entries
     int ndir[3];               // directions of entry k
     int dx[3][3], dy[3][3];
     int plane[3][3];           // their output planes, numbered in this order
     int nlines[3];
     int jbegin[4];
-    int nlong;                   // jobs [0, nlong) belong to the long-axis directions
-    uint32_t unit;               // always 1; see the kernel's multiply-adds
+    int klong;                 // entry of the long-axis directions (-1: none)
+    int nlong;                 // their jobs
+    uint32_t unit;             // always 1; see the kernel's multiply-adds
 };
 
 // Work-queue state of the aggregation kernel: word 0 counts the jobs handed out
 // beyond the warps' first ones (cleared before every launch).
 constexpr size_t kJobStateBytes = 4224;
 
-// Builds the work list for the directions in `mask`, longest scanlines first, under the
+// Builds the work list for the directions in `mask`, under the
 // sgm_set_aggregation setting cpl.  many: other pairs' work runs beside it, so
-// the lanes are not narrowed to shorten a small image's chains.
+// the lanes are not narrowed to shorten a small image's chains and the long axis
+// comes first.
 PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool many = false);
 // Resident 4-warp blocks per SM for a handle whose caller sets none.
 int default_blocks_per_sm(const PathJobs &jobs);

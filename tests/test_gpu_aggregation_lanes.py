@@ -36,3 +36,22 @@ def test_lane_widths_match_the_oracle(W, H, D, turn):
         h.compute(L, R, disp)
         assert np.array_equal(S.cpu().numpy().view(np.uint16), o["S"])
         assert np.array_equal(disp.cpu().numpy(), o["disp"])
+
+
+@pytest.mark.parametrize("W, H", [(700, 560), (560, 700)])
+def test_costs_beyond_l2_match_the_oracle(W, H):
+    # 16-bit costs of 100 MB: the long axis is walked between the two sweeps
+    rng = np.random.default_rng(W)
+    left = rng.integers(0, 256, (H, W), dtype=np.uint8)
+    right = np.roll(left, -40, axis=1)
+    p = sgm.SgmParams(census_w=3, census_h=3, path_mask=0xFF, P1=200, P2=800, lr_tolerance=1, median_k=3,
+                      cost=sgm.SGM_COST_SAD)
+    o = oracle.sgm(left, right, 128, 3, 3, 0xFF, 200, 800, 1, 3, stages=True, uv=False, cost=sgm.SGM_COST_SAD)
+    with sgm.Handle(W, H, 128, p) as h:
+        disp = torch.empty((H, W), dtype=torch.uint8, device="cuda")
+        S = torch.empty((H, W, 128), dtype=torch.int16, device="cuda")
+        L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+        sgm.sgm_debug_sum(h, L, R, S)
+        h.compute(L, R, disp)
+        assert np.array_equal(S.cpu().numpy().view(np.uint16), o["S"])
+        assert np.array_equal(disp.cpu().numpy(), o["disp"])
