@@ -103,6 +103,11 @@ constexpr int kSchedulers = 608;  // warp schedulers of the GPU (152 SMs)
 //   D = 32    246 x 269, 8 paths: base 25.5, (1, 1) 18.7;  1280 x 720: base 123.9, (1, 4) 132.9
 //   D = 128   230 x 182, 8 paths: base 22.2, (2, 2) 19.5;  480 x 752: base 97.5, (2, 2) 104
 //
+// Four paths at D = 128 also take (2, 2) where the base leaves a second round of jobs
+// nearly empty (rounds of 16 warps per SM, base): 1.03 (800 x 900) base 127, (2, 2) 107;
+// 1.12 (1280 x 720) 154, 142;  1.15 (1400 x 700) 162, 143;  1.30 (1044 x 1079) 205, 181;
+// 1.42 (1300 x 1080) 235, 239;  0.92 (708 x 818) 88, 94.
+//
 // 96 and 192 slots are 12 or 24 lanes of four pairs, which leave a quarter of every
 // warp idle; 8 or 16 lanes of six fill it.  It pays where the diagonals read their
 // costs from L2 and the warps, fewer by a third, still fill the chip:
@@ -138,7 +143,11 @@ LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool m
         if (warps(1, 4) <= 4 * kSchedulers) return {1, 4};
         return lc;
     }
-    if (Dp <= 128 && 50. * shorter > 31. * longer && warps(2, 2) <= 4 * kSchedulers) lc.np_other = 2;
+    // without diagonals, base warps that fill a second round of 16 per SM by a third at most
+    const long base = warps(lc.np_long, 4);
+    const bool both = (mask & (0x0F ^ axis)) == (0x0F ^ axis) && !(mask & 0xF0);
+    const bool short_round = Dp == 128 && both && base > 4 * kSchedulers && base <= 5.4 * kSchedulers;
+    if (short_round || (Dp <= 128 && 50. * shorter > 31. * longer && warps(2, 2) <= 4 * kSchedulers)) lc.np_other = 2;
     else if (!wide && Dp % 96 == 0 && (mask & 0xF0) && warps(lc.np_long, 6) >= 3 * kSchedulers) lc.np_other = 6;
     return lc;
 }
