@@ -908,7 +908,7 @@ cudaError_t launch_aggregate_batch(const BatchAggPair *pairs, int npairs, const 
     const size_t smem = kWarps * kRingBytes + sizeof(int) * 2 * (size_t)(npairs + 1);
     auto kernel = wide ? aggregate_batch_kernel<1, true>
                        : cpl == 4 ? aggregate_batch_kernel<4, false> : aggregate_batch_kernel<1, false>;
-    const cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t ea = allow_max_smem(kernel);
     if (ea != cudaSuccess) return ea;
     return launch_k(kernel, dim3(blocks), dim3(kWarps * 32), smem, s, pairs, npairs, prefix, P1x2, P2x2, job_counter, sms);
 }

@@ -306,9 +306,8 @@ cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch
                         ((srows * rcols + 3) & ~(size_t)3) + srows * rcols * 4;
     const dim3 grid((W + kSeg - 1) / kSeg, (H + kRows - 1) / kRows);
     uint4 *out = reinterpret_cast<uint4 *>(cost);
-    cudaError_t e;
     auto kernel = maps.lx ? sad_cost_kernel<true> : sad_cost_kernel<false>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_max_smem(kernel);
     if (e != cudaSuccess) return e;
     return launch_k(kernel, grid, dim3(kThreads), smem, s, left, right, pitch, W, H, D, Dp, ww, wh, maps, out,
                     job_state);

@@ -56,6 +56,16 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Lets a kernel that declares no shared memory of its own have all a CTA can have.
+// The limit belongs to the function on the device, not to the launch: always the
+// same value, as one that followed the launch's size could be lowered by another
+// host thread before the launch.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <typename... KArgs>
+cudaError_t allow_max_smem(void (*kernel)(KArgs...)) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 struct RectMaps {
     const uint16_t *lx, *ly, *rx, *ry;
 };

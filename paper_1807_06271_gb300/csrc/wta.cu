@@ -260,10 +260,10 @@ size_t wta_smem_bytes(int W, int Dp, size_t rec, int warps) {
     return (size_t)warps * kStages * rec + (size_t)(Dp + W) * sizeof(uint32_t) + (size_t)((W + 3) & ~3);
 }
 
-// As many warps as fit a CTA's 227 KB.
+// As many warps as fit a CTA's shared memory.
 int wta_warps(int W, int Dp, size_t rec) {
     int warps = kMaxWarps;
-    while (warps > 1 && wta_smem_bytes(W, Dp, rec, warps) > 227 * 1024) warps /= 2;
+    while (warps > 1 && wta_smem_bytes(W, Dp, rec, warps) > kMaxSmem) warps /= 2;
     return warps;
 }
 
@@ -275,7 +275,7 @@ cudaError_t launch_wta_t(const uint8_t *planes, int nplanes, int W, int H, int D
     const bool all = warps == kMaxWarps;
     auto go = [&](auto kernel, int G) {
         const size_t smem = wta_smem_bytes(W, Dp, (size_t)G * nplanes * Dp * (WIDE ? 2 : 1), warps);
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_max_smem(kernel);
         if (e != cudaSuccess) return e;
         return launch_k(kernel, dim3(H), dim3(warps * 32), smem, s, planes, nplanes, W, H, D, Dp, tol, disp_lr, dbg_left,
                         dbg_right, dbg_sum);
