@@ -383,7 +383,7 @@ int sgm_debug_stalled_wait(sgm_handle h, const uint8_t *left, const uint8_t *rig
 
 /* Guarded builds only (the library compiled with -DSGM_GUARDED, which
  * paper_1807_06271_gb300.build makes as libsgm_guarded.so for tests; the
- * paper has no counterpart).  In them the census, CUDA-core cost,
+ * paper has no counterpart).  In them the census, CUDA-core cost, SAD cost,
  * aggregation, WTA, median and U/V kernels check every global index they
  * compute, and every image-dependent shared-memory index, against the
  * buffer's extent, skip an access out of range and count it.  Writes to

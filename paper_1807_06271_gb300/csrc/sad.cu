@@ -152,13 +152,14 @@ __global__ void __launch_bounds__(kThreads)
         __syncthreads();
         // Quarter q of a record: pairs 4q + e = disparities (4q + e, Dp-1-4q-e), e < 4:
         // half q % 2 of the chunk q / 2, and the other half of its mirror image backwards.
-        uint4 *out = cost + ((size_t)(y0 + r) * W + x0) * chunks;
+        const long long at = ((long long)(y0 + r) * W + x0) * chunks;
         for (int it = threadIdx.x; it < npx * chunks; it += kThreads) {
+            if (!in_range(at + it, (long long)W * H * chunks)) continue;
             const int px = it / chunks, q = it - px * chunks;
             const uint4 l = tile[px * chunks + (q >> 1)], h = tile[px * chunks + chunks - 1 - (q >> 1)];
             const uint32_t sel = q & 1 ? 0x5432u : 0x7610u;
-            out[it] = make_uint4(__byte_perm(l.x, h.w, sel), __byte_perm(l.y, h.z, sel), __byte_perm(l.z, h.y, sel),
-                                 __byte_perm(l.w, h.x, sel));
+            cost[at + it] = make_uint4(__byte_perm(l.x, h.w, sel), __byte_perm(l.y, h.z, sel), __byte_perm(l.z, h.y, sel),
+                                       __byte_perm(l.w, h.x, sel));
         }
     }
 }
@@ -285,6 +286,8 @@ __global__ void __launch_bounds__(128)
 }
 
 }  // namespace
+
+SGM_GUARD_COUNTER(guard_hits_sad)
 
 cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch, int W, int H,
                             int D, int ww, int wh, const RectMaps &maps, uint16_t *cost,

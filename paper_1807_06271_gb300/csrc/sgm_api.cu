@@ -672,7 +672,7 @@ int sgm_debug_guard_hits(unsigned long long *hits, int reset) {
     if (!hits) return SGM_ERR_INVALID_ARG;
 #ifdef SGM_GUARDED
     unsigned long long total = 0;
-    for (unsigned long long v : {guard_hits_census(reset != 0), guard_hits_aggregate(reset != 0),
+    for (unsigned long long v : {guard_hits_census(reset != 0), guard_hits_sad(reset != 0), guard_hits_aggregate(reset != 0),
                                  guard_hits_wta(reset != 0), guard_hits_post(reset != 0)}) {
         if (v == ~0ull) {
             cudaGetLastError();

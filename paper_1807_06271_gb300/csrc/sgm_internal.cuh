@@ -74,8 +74,8 @@ struct RectMaps {
 // maps (Sec. 3.1.1), 0 where a map entry leaves the source.
 // Guarded builds (compiled with -DSGM_GUARDED: a test variant of the
 // library, never the default).  The plane path's kernels (census, the
-// CUDA-core cost, the aggregation, the WTA, the median and the U/V maps)
-// check each global index they compute, and each shared index that depends
+// CUDA-core and SAD costs, the aggregation, the WTA, the median and the U/V
+// maps) check each global index they compute, and each shared index that depends
 // on the image, against its buffer's extent before the access.  An index out
 // of range skips the access and is counted in the translation unit's
 // counter; sgm_debug_guard_hits sums the counters.  In the default build
@@ -103,6 +103,7 @@ __device__ __forceinline__ constexpr bool in_range(long long, long long) { retur
 #endif
 // Each guarded translation unit's counter (~0 when it cannot be read).
 unsigned long long guard_hits_census(bool reset);
+unsigned long long guard_hits_sad(bool reset);
 unsigned long long guard_hits_aggregate(bool reset);
 unsigned long long guard_hits_wta(bool reset);
 unsigned long long guard_hits_post(bool reset);
