@@ -307,7 +307,8 @@ int sgm_get_shape(sgm_handle h, int *W, int *H, int *D, int *census_bits);
  * disparities and `params` (checked as by sgm_create; the paper has no
  * counterpart).  *handle_bytes: what sgm_create allocates (census codes, cost
  * volume, one plane per enabled path, LR map, work-queue state), without the
- * guard bytes of sgm_debug_canaries.  *host_staging_bytes: what the
+ * guard bytes of sgm_debug_canaries; a pixel of the cost volume or of a plane
+ * owns 8, 16 or the multiple of 32 slots that holds D.  *host_staging_bytes: what the
  * host-buffer entry points add on their first use (two staging slots of
  * left, right, disp, U and V).  *static_bytes: the part of the fixed array
  * that sgm_compute_static would use (it runs only when this is at most

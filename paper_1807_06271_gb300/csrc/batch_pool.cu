@@ -323,7 +323,7 @@ int sgm_batch_create(int n, const int *W, const int *H, const int *D, const sgm_
         ps.H = H[i];
         ps.D = D[i];
         ps.Dp = padded_disparities(D[i]);
-        const ScratchSizes sz = scratch_sizes(W[i], H[i], D[i], params);
+        const ScratchSizes sz = scratch_sizes(W[i], H[i], D[i], params, ps.Dp);
         ps.codes = at;
         at = align256(at + sz.codes);
         ps.cost = at;

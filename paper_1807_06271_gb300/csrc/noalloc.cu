@@ -106,7 +106,8 @@ struct DeviceSwitch {
 
 }  // namespace
 
-sgm::StaticLayout sgm::static_layout(const ScratchSizes &sz) {
+sgm::StaticLayout sgm::static_layout(int W, int H, int D, const sgm_params *p) {
+    const ScratchSizes sz = scratch_sizes(W, H, D, p, 8 * lanes_per_scanline(D));
     StaticLayout l;
     l.codes = 0;
     l.cost = round_up(l.codes + sz.codes, 256);
@@ -123,8 +124,7 @@ extern "C" int sgm_compute_static(int W, int H, int D, const sgm_params *params,
     if (!left || !right || !disp) return SGM_ERR_INVALID_ARG;
     int rc = sgm::validate_params(W, H, D, params);
     if (rc != SGM_OK) return rc;
-    const sgm::ScratchSizes sz = sgm::scratch_sizes(W, H, D, params);
-    const sgm::StaticLayout at = sgm::static_layout(sz);
+    const sgm::StaticLayout at = sgm::static_layout(W, H, D, params);
     if (at.end > (size_t)SGM_STATIC_SCRATCH_BYTES) return SGM_ERR_UNSUPPORTED;
 
     // The three buffers must be device memory of one device; the call runs on

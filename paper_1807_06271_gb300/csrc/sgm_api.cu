@@ -276,12 +276,12 @@ int sgm::compute_pair(sgm_handle_s *h, const uint8_t *left, const uint8_t *right
 // Same host-side argument checks as sgm_create, for entry points without a handle.
 int sgm::validate_params(int W, int H, int D, const sgm_params *p) { return validate(W, H, D, p); }
 
-sgm::ScratchSizes sgm::scratch_sizes(int W, int H, int D, const sgm_params *p) {
+sgm::ScratchSizes sgm::scratch_sizes(int W, int H, int D, const sgm_params *p, int slots) {
     const bool wide = p->cost == SGM_COST_SAD;
     const int nbits = p->census_w * p->census_h - 1;
     const size_t code_bytes = wide ? 0 : (nbits <= 32 ? 4 : 8);
     const size_t eb = wide ? 2 : 1;  // bytes per cost / path cost
-    const size_t npx = (size_t)W * H, Dp = (size_t)scratch_disparities(D);
+    const size_t npx = (size_t)W * H, Dp = (size_t)slots;
     const size_t npaths = (size_t)__builtin_popcount((unsigned)p->path_mask);
     ScratchSizes s;
     s.codes = 2 * npx * code_bytes;
@@ -355,7 +355,7 @@ int sgm_create(int W, int H, int D, const sgm_params *params, sgm_handle *out) {
         const int v = atoi(env);
         if (v >= 1 && v <= 16) h->agg_blocks_per_sm = v;
     }
-    const ScratchSizes sz = scratch_sizes(W, H, D, params);
+    const ScratchSizes sz = scratch_sizes(W, H, D, params, h->Dp);
     h->canaries = g_canaries.load();
     rc = h->wide ? SGM_OK : dev_alloc(h, &h->codes, sz.codes);
     if (rc == SGM_OK) rc = dev_alloc(h, &h->cost, sz.cost);
@@ -396,10 +396,10 @@ int sgm_scratch_bytes(int W, int H, int D, const sgm_params *params, size_t *han
                       size_t *host_staging_bytes, size_t *static_bytes) {
     const int rc = validate(W, H, D, params);
     if (rc != SGM_OK) return rc;
-    const ScratchSizes sz = scratch_sizes(W, H, D, params);
+    const ScratchSizes sz = scratch_sizes(W, H, D, params, padded_disparities(D));
     if (handle_bytes) *handle_bytes = sz.handle();
     if (host_staging_bytes) *host_staging_bytes = 2 * sz.staging_slot;
-    if (static_bytes) *static_bytes = static_scratch_bytes(sz);
+    if (static_bytes) *static_bytes = static_layout(W, H, D, params).end;
     return SGM_OK;
 }
 

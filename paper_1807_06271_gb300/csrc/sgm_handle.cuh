@@ -87,9 +87,10 @@ struct sgm_handle_s {
 
 namespace sgm {
 
-// Bytes of each device buffer of one pair.  sgm_create allocates each as its
-// own buffer, sgm_compute_static packs them into its fixed array, and
-// sgm_scratch_bytes reports them, all from this one computation.
+// Bytes of each device buffer of one pair whose pixels own `slots` slots.
+// sgm_create allocates each as its own buffer, sgm_compute_static packs them into
+// its fixed array, and sgm_scratch_bytes reports them, all from this one
+// computation.
 struct ScratchSizes {
     size_t codes;         // census codes of both images (0 for SAD)
     size_t cost;          // cost volume
@@ -101,16 +102,17 @@ struct ScratchSizes {
     size_t handle() const { return codes + cost + job_state + planes + disp_lr + sweep; }
 };
 // Call only with parameters that passed validate_params.
-ScratchSizes scratch_sizes(int W, int H, int D, const sgm_params *p);
+ScratchSizes scratch_sizes(int W, int H, int D, const sgm_params *p, int slots);
 
 // Where sgm_compute_static places each buffer in its fixed array: codes,
 // cost volume, planes, work-queue state and LR map in turn, each at a
-// 256-byte boundary; end is the number of bytes used.
+// 256-byte boundary; end is the number of bytes used.  Volumes have room for a
+// power of two of slots, the layout that sgm.h documents and by which the call
+// takes or refuses a shape; the kernels use padded_disparities(D) of them.
 struct StaticLayout {
     size_t codes, cost, planes, job_state, disp_lr, end;
 };
-StaticLayout static_layout(const ScratchSizes &sz);
-inline size_t static_scratch_bytes(const ScratchSizes &sz) { return static_layout(sz).end; }
+StaticLayout static_layout(int W, int H, int D, const sgm_params *p);
 
 // One pair (and its U/V maps when umap and vmap are non-null) on stream s.
 int compute_pair(sgm_handle_s *h, const uint8_t *left, const uint8_t *right, uint8_t *disp,

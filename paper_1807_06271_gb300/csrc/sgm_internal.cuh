@@ -143,8 +143,6 @@ inline int lanes_per_scanline(int D) {  // 8-disparity chunks of D, rounded up t
 inline int padded_disparities(int D) {
     return D <= 8 ? 8 : D <= 16 ? 16 : (D + 31) / 32 * 32;
 }
-// Disparities that scratch buffers are sized for (a power of two, at least Dp).
-inline int scratch_disparities(int D) { return 8 * lanes_per_scanline(D); }
 // Slot (byte, or uint16 for wide) of disparity d in a pixel's record.
 __host__ __device__ constexpr int fold_slot(int d, int Dp, bool wide) {
     const int hi = d >= Dp / 2, k = hi ? Dp - 1 - d : d;
