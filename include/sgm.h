@@ -242,9 +242,10 @@ int sgm_batch_device_bytes(sgm_batch b, size_t *bytes);
  * one chunk, or half of one on the long-axis scanlines (rows when W >= H) while
  * D <= 128, whose chain of steps sets the kernel's duration, and down to a
  * quarter of one on small images (D = 65 to 96 and 161 to 192 may take one and a
- * half); with 2 and 4 it holds that many chunks in
- * every direction, and MIXED is one chunk on the long-axis scanlines and two
- * in the other directions (where D spans a power of two of chunks; else as 1).
+ * half); with 2 and 4 it holds that many chunks in every direction, and MIXED is
+ * one chunk on the long-axis scanlines and two in the other directions.  For D =
+ * 65 to 96 and 129 to 224, whose slots are no power of two, 2, 4 and MIXED are
+ * taken and reported as set and run as 1.
  * SGM_ERR_UNSUPPORTED above what D allows (D must span at least that many
  * chunks; the 16-bit costs of SGM_COST_SAD take 1).  More disparities per lane
  * let a warp walk more scanlines at once with fewer instructions per
@@ -285,11 +286,11 @@ int sgm_set_schedule(sgm_handle h, int schedule, int rows_per_cta);
 int sgm_get_schedule(sgm_handle h, int *schedule, int *rows_per_cta);
 
 /* Autotuner: times the pipeline on this pair (device pointers as for
- * sgm_compute; disp is overwritten) with the PLANES schedule at 1, 2, 3, 4
- * and 6 resident aggregation blocks per SM, each with 1, 2 and 4 chunks per
- * lane and the mixed layout where D allows (sgm_set_aggregation), and, where
- * h can run it, the SWEEP
- * schedule at 2, 4 and 8 rows per block; keeps the fastest for h and for
+ * sgm_compute; disp is overwritten) with the PLANES schedule at h's own
+ * aggregation setting, at the one a new handle of this shape starts with, and at
+ * 1, 2, 3, 4 and 6 resident blocks per SM, each with 1, 2 and 4 chunks per lane
+ * and the mixed layout where D takes them (sgm_set_aggregation), and, where h
+ * can run it, the SWEEP schedule at 2, 4 and 8 rows per block; keeps the fastest for h and for
  * handles created later in this process with the same W, H, D, path mask,
  * cost, window and P2.  *best_blocks_per_sm (may be NULL) receives the best
  * PLANES setting; sgm_get_schedule tells which schedule won.  Synchronises

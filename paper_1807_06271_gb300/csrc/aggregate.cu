@@ -116,10 +116,11 @@ constexpr int kSchedulers = 608;  // warp schedulers of the GPU (152 SMs)
 //   D = 96    1784 x 799, 8 paths: (2, 4) 486, (2, 6) 460;  640 x 480: 86, 98
 LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool many) {
     const int Dp = padded_disparities(D);
-    const bool pow2 = (Dp & (Dp - 1)) == 0;  // lanes of more than 4 pairs come in powers of two
-    if (!wide && pow2 && cpl == 2) return {8, 8};
-    if (!wide && pow2 && cpl == 4) return {16, 16};
-    if (!wide && pow2 && cpl == kMixedCpl) return {4, 8};
+    if (chunks_apply(D, wide)) {
+        if (cpl == 2) return {8, 8};
+        if (cpl == 4) return {16, 16};
+        if (cpl == kMixedCpl) return {4, 8};
+    }
     LaneConfig lc{Dp <= 128 ? 2 : 4, 4};
     if (many || Dp < 32) return lc;
     const int axis = W >= H ? 0x03 : 0x0C;  // the long-axis directions
@@ -870,6 +871,11 @@ cudaError_t sm_count(int *sms) {
 }
 
 }  // namespace
+
+bool chunks_apply(int D, bool wide) {
+    const int Dp = padded_disparities(D);
+    return !wide && (Dp & (Dp - 1)) == 0;  // lanes of 8 and 16 pairs come in powers of two
+}
 
 int chunks_per_lane_max(int D, bool wide) {
     const int chunks = lanes_per_scanline(D);  // 8-disparity chunks per pixel

@@ -191,6 +191,9 @@ PathJobs make_path_jobs(int W, int H, int D, int mask, bool wide, int cpl, bool 
 int default_blocks_per_sm(const PathJobs &jobs);
 // The most chunks per lane the aggregation takes for D (1 for 16-bit costs, up to 4).
 int chunks_per_lane_max(int D, bool wide);
+// Whether the settings above 1 change the lanes for D (they run as 1 for 96, 160, 192
+// and 224 slots).
+bool chunks_apply(int D, bool wide);
 // Chunks-per-lane code of the mixed layout: long-axis scanlines at 1, the others at 2.
 constexpr int kMixedCpl = SGM_AGG_CHUNKS_MIXED;
 
