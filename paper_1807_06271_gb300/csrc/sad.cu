@@ -19,10 +19,10 @@
 // that leaves).  |a - b| = max.u16x2 - min.u16x2 (full rate on GB300).
 // Each row's costs then add ww neighbouring columns of V, four packed adds
 // per chunk and column (halves never carry: a cost is at most
-// ww * wh * 255 <= 32766).  The chunks go through a shared tile, from which
-// each 16-byte quarter of a folded record takes the halves of two chunks
-// from either end of the disparity range; consecutive threads write
-// consecutive quarters of the segment's contiguous pixel records.
+// ww * wh * 255 <= 32766).  A thread sums a chunk and its mirror image at the
+// other end of the disparity range, whose halves make up two 16-byte quarters of
+// the pixel's folded record; consecutive threads write consecutive 32 bytes of the
+// segment's contiguous records.
 #include "sgm_internal.cuh"
 
 namespace sgm {
@@ -31,6 +31,14 @@ namespace {
 // 64 pixels x 4 rows per CTA: rows per CTA against threads measured on GB300
 // (640 x 360, D = 60, 5 x 5): 8 rows 29.0 us, 16 rows 38.3, 2 rows (128
 // threads) 29.0, 4 rows 27.0 us; more CTAs hide the row staging better.
+//
+// Bound by instruction issue and shared memory.  Two chunks per thread and the
+// vertical sums in mirror order fold the records for nothing: chunks through a
+// shared tile, then the records from it, and this, us: 1242 x 375, D = 128, 3 x 3
+// 81.8, 70.0, 7 x 7 112.4, 101.0; 640 x 360, D = 60, 3 x 3 28.6, 24.6; 1280 x 720, D =
+// 96, 7 x 7 139.3, 127.0 (chunks in their natural order 153.9: bank conflicts); halves
+// exchanged between lanes 76.4, 103.6, 28.6, 133.2.  The column loop is not unrolled:
+// with 54 registers instead of 40 four CTAs fit an SM instead of six (640 x 360 26.8).
 constexpr int kSeg = 64, kRows = 4, kThreads = 256;
 
 __device__ __forceinline__ uint32_t vmin2(uint32_t a, uint32_t b) {
@@ -64,6 +72,18 @@ __device__ __forceinline__ void absdiff_row(uint4 &v, uint32_t l, const uint32_t
     }
 }
 
+// The chunk at place r of a column's vertical sums: mirror images side by side (an
+// even number of chunks, or one).
+__device__ __forceinline__ int chunk_at(int r, int chunks) { return r & 1 ? chunks - 1 - (r >> 1) : r >> 1; }
+
+// The pair of costs of the disparities (d, d + 4) at column x, with the padding and
+// the columns left of the image put in.
+__device__ __forceinline__ uint32_t edge_pair(uint32_t v, int d, int x, int D, uint32_t cmax) {
+    const uint32_t lo = d >= D ? kPadCostWide : x - d < 0 ? cmax : (v & 0xFFFFu);
+    const uint32_t hi = d + 4 >= D ? kPadCostWide : x - d - 4 < 0 ? cmax : (v >> 16);
+    return lo | (hi << 16);
+}
+
 template <bool RECT>
 __global__ void __launch_bounds__(kThreads)
     sad_cost_kernel(const uint8_t *__restrict__ left, const uint8_t *__restrict__ right, int pitch,
@@ -75,13 +95,12 @@ __global__ void __launch_bounds__(kThreads)
     const int rw = ww / 2, rh = wh / 2;
     const int ncol = kSeg + 2 * rw;          // V columns (segment + halo)
     const int lcols = ncol, rcols = kSeg + Dp - 1 + 2 * rw;
-    const int chunks = Dp / 8;
+    const int chunks = Dp / 8, mirrored = (chunks + 1) / 2;  // an even number of chunks, or one
     const int y0 = blockIdx.y * kRows, x0 = blockIdx.x * kSeg;
     const int nrows = min(kRows, H - y0);   // output rows of this CTA
     const int srows = nrows + wh - 1;       // staged rows: y0 - rh .. y0 + nrows - 1 + rh
-    uint4 *V = reinterpret_cast<uint4 *>(sad_smem);                              // [ncol][chunks]
-    uint4 *tile = V + (size_t)ncol * chunks;                                      // [kSeg][chunks] costs of a row
-    uint32_t *Lp = reinterpret_cast<uint32_t *>(tile + (size_t)kSeg * chunks);   // [srows][lcols]: (l, l)
+    uint4 *V = reinterpret_cast<uint4 *>(sad_smem);                              // [ncol][chunks], chunk_at order
+    uint32_t *Lp = reinterpret_cast<uint32_t *>(V + (size_t)ncol * chunks);      // [srows][lcols]: (l, l)
     uint8_t *Rb = reinterpret_cast<uint8_t *>(Lp + srows * lcols);               // [srows][rcols] bytes
     uint32_t *Rp = reinterpret_cast<uint32_t *>(Rb + ((srows * rcols + 3) & ~3));  // [srows][rcols]: (R[c], R[c-4])
     const int xl0 = x0 - rw;            // image column of left column 0
@@ -111,7 +130,7 @@ __global__ void __launch_bounds__(kThreads)
         // of chunk (j, i) reads the right pair at c0 - k, c0 = j + Dp - 1 - 8i:
         // column j - d + Dp - 1 for d = 8i + k, high half 4 columns left (>= j >= 0).
         for (int it = threadIdx.x; it < ncol * chunks; it += kThreads) {
-            const int j = it / chunks, i = it - j * chunks;
+            const int j = it / chunks, i = chunk_at(it - j * chunks, chunks);
             const int c0 = j + Dp - 1 - 8 * i;
             uint4 v;
             if (r == 0) {
@@ -126,41 +145,52 @@ __global__ void __launch_bounds__(kThreads)
             V[it] = v;
         }
         __syncthreads();
-        // C(x, d) = sum over u < ww of V(x - x0 + u, d); cmax where x - d < 0.
-        for (int it = threadIdx.x; it < npx * chunks; it += kThreads) {
-            const int px = it / chunks, i = it - px * chunks;
-            uint32_t s[4] = {0u, 0u, 0u, 0u};
-            for (int u = 0; u < ww; u++) {
-                const uint4 q = V[(px + u) * chunks + i];
-                s[0] += q.x;
-                s[1] += q.y;
-                s[2] += q.z;
-                s[3] += q.w;
+        // C(x, d) = sum over u < ww of V(x - x0 + u, d); cmax where x - d < 0.  A thread
+        // sums chunk i and its mirror image m = chunks - 1 - i, whose halves make up the
+        // quarters 2i and 2i + 1 of the pixel's record: the pairs 8i + e, e < 4, hold the
+        // lower halves of i and the upper ones of m backwards, the pairs 8i + 4 + e what
+        // remains.  Half of the lanes read m first, so that the lanes read distinct banks.
+        const long long at = ((long long)(y0 + r) * W + x0) * chunks;
+        const int mfirst = chunks > 1 && (threadIdx.x & 4) ? 1 : 0, step = chunks > 1 ? 1 - 2 * mfirst : 0;
+        for (int it = threadIdx.x; it < npx * mirrored; it += kThreads) {
+            const int px = it / mirrored, i = it - px * mirrored;
+            const uint4 *v = V + px * chunks + 2 * i + mfirst;
+            uint32_t a[4] = {0u, 0u, 0u, 0u}, b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+            for (int u = 0; u < ww; u++, v += chunks) {
+                const uint4 p = v[0], q = v[step];
+                a[0] += p.x;
+                a[1] += p.y;
+                a[2] += p.z;
+                a[3] += p.w;
+                b[0] += q.x;
+                b[1] += q.y;
+                b[2] += q.z;
+                b[3] += q.w;
+            }
+            uint32_t l[4], m[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                l[k] = mfirst ? b[k] : a[k];
+                m[k] = mfirst ? a[k] : b[k];
             }
             if (ragged || border) {
-                const int x = x0 + px;
+                const int x = x0 + px, dm = Dp - 8 - 8 * i;
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
-                    const int dlo = 8 * i + k, dhi = dlo + 4;
-                    const uint32_t vlo = dlo >= D ? kPadCostWide : x - dlo < 0 ? cmax : (s[k] & 0xFFFFu);
-                    const uint32_t vhi = dhi >= D ? kPadCostWide : x - dhi < 0 ? cmax : (s[k] >> 16);
-                    s[k] = vlo | (vhi << 16);
+                    l[k] = edge_pair(l[k], 8 * i + k, x, D, cmax);
+                    m[k] = edge_pair(m[k], dm + k, x, D, cmax);
                 }
             }
-            tile[it] = make_uint4(s[0], s[1], s[2], s[3]);
+            const long long o = at + px * chunks + 2 * i;
+            if (in_range(o, (long long)W * H * chunks))
+                cost[o] = make_uint4(__byte_perm(l[0], m[3], 0x7610), __byte_perm(l[1], m[2], 0x7610),
+                                     __byte_perm(l[2], m[1], 0x7610), __byte_perm(l[3], m[0], 0x7610));
+            if (chunks > 1 && in_range(o + 1, (long long)W * H * chunks))
+                cost[o + 1] = make_uint4(__byte_perm(l[0], m[3], 0x5432), __byte_perm(l[1], m[2], 0x5432),
+                                         __byte_perm(l[2], m[1], 0x5432), __byte_perm(l[3], m[0], 0x5432));
         }
         __syncthreads();
-        // Quarter q of a record: pairs 4q + e = disparities (4q + e, Dp-1-4q-e), e < 4:
-        // half q % 2 of the chunk q / 2, and the other half of its mirror image backwards.
-        const long long at = ((long long)(y0 + r) * W + x0) * chunks;
-        for (int it = threadIdx.x; it < npx * chunks; it += kThreads) {
-            if (!in_range(at + it, (long long)W * H * chunks)) continue;
-            const int px = it / chunks, q = it - px * chunks;
-            const uint4 l = tile[px * chunks + (q >> 1)], h = tile[px * chunks + chunks - 1 - (q >> 1)];
-            const uint32_t sel = q & 1 ? 0x5432u : 0x7610u;
-            cost[at + it] = make_uint4(__byte_perm(l.x, h.w, sel), __byte_perm(l.y, h.z, sel), __byte_perm(l.z, h.y, sel),
-                                       __byte_perm(l.w, h.x, sel));
-        }
     }
 }
 
@@ -173,12 +203,25 @@ __global__ void __launch_bounds__(kThreads)
 // sums of its kRows5 output rows (each the one above plus the row entering minus
 // the row leaving), and adds the last four columns' sums, which it keeps.
 // Bound by instruction issue (about 55 a column, row and quarter); the kernel
-// above goes through shared memory and three barriers per row for the same
+// above goes through shared memory and two barriers per row for the same
 // sums.  kSegLen is 3 modulo 4 so that the segments of a warp read distinct banks.
-// Measured, us, against the kernel above: 640 x 360, D = 60: 30.3 -> 22.2; 1242 x 375,
-// D = 128: 94.6 -> 55.5; 430 x 312, D = 192: 63 -> 33; 320 x 240, D = 64: 16.6 -> 16.6.
-// 4 rows took 27.0 / 68.0 / 41.1 / 20.7, segments of 31 pixels 37 / 58.8 / 37.2 / 23.5.
+// Measured, us, the kernel above and this one: 640 x 360, D = 60: 26.9, 21.2; 1242 x
+// 375, D = 128: 85.8, 55.6; 430 x 312, D = 192: 52.1, 32.8.  4 rows took 27.0 / 68.0 /
+// 41.1, segments of 31 pixels 37 / 58.8 / 37.2.
 constexpr int kRows5 = 2, kSegLen = 15;
+
+// Whether a W x H image with Dp slots takes this kernel.  With few slots its CTAs are
+// wide, and a small image has too few of them.  Measured, us, the kernel above and
+// this one:
+//   8 to 32 slots  320 x 240 (D = 16) 10.5, 17.0;  640 x 480 22.6, 25.1;  800 x 600 32.2, 25.6;
+//                  1280 x 720 51.4, 47.2, (D = 16) 36.9, 37.0;  640 x 480 (D = 8) 16.5, 18.6
+//   64 slots       320 x 240 14.6, 16.6;  350 x 250 16.5, 16.4;  300 x 300 16.4, 16.4;
+//                  240 x 480 20.6, 16.5;  480 x 260 20.6, 16.7
+//   more           160 x 96 (D = 96) 15.5, 14.1;  100 x 40 (D = 128) 16.4, 13.4
+bool window5_pays(int W, int H, int Dp) {
+    const long npx = (long)W * H;
+    return Dp >= 96 || npx >= (Dp == 64 ? 90000 : 400000);
+}
 
 template <bool RECT>
 __global__ void __launch_bounds__(128)
@@ -295,7 +338,7 @@ cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch
     if (ww < 1 || wh < 1 || ww > kMaxSadWindow || wh > kMaxSadWindow)
         return cudaErrorInvalidValue;
     const int Dp = padded_disparities(D);
-    if (ww == 5 && wh == 5) {
+    if (ww == 5 && wh == 5 && window5_pays(W, H, Dp)) {
         const int segs = Dp < 32 ? 32 : 128 / (Dp / 8), width = segs * kSegLen;
         const size_t smem = (size_t)(kRows5 + 4) * (2 * (width + 8) + Dp) * sizeof(uint32_t);
         return launch_k(maps.lx ? sad5_cost_kernel<true> : sad5_cost_kernel<false>,
@@ -305,7 +348,7 @@ cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch
     const int rw = ww / 2;
     const int ncol = kSeg + 2 * rw, rcols = kSeg + Dp - 1 + 2 * rw;
     const size_t srows = (size_t)kRows + wh - 1;
-    const size_t smem = (size_t)(ncol + kSeg) * (Dp / 8) * sizeof(uint4) + srows * ncol * 4 +
+    const size_t smem = (size_t)ncol * (Dp / 8) * sizeof(uint4) + srows * ncol * 4 +
                         ((srows * rcols + 3) & ~(size_t)3) + srows * rcols * 4;
     const dim3 grid((W + kSeg - 1) / kSeg, (H + kRows - 1) / kRows);
     uint4 *out = reinterpret_cast<uint4 *>(cost);

@@ -28,6 +28,7 @@ CASES = [
     (77, 30, 130, CENSUS, (7, 5), 0xFF, 8, 64, False),   # 160 slots
     (50, 33, 200, CENSUS, (3, 3), 0x55, 8, 64, False),   # 224 slots
     (61, 20, 60, SAD, (5, 5), 0x55, 200, 800, False),
+    (481, 188, 60, SAD, (5, 5), 0x55, 200, 800, False),
     (130, 11, 96, SAD, (5, 5), 0xFF, 200, 800, True),
     (67, 13, 3, SAD, (7, 7), 0x0F, 200, 800, False),
     (129, 9, 100, SAD, (3, 3), 0xFF, 200, 800, True),
