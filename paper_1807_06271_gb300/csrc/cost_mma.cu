@@ -28,9 +28,9 @@
 // convert segment k, the MMAs of k+1 run and every thread holds its share of
 // the codes of k+2.
 //
-// Standing.  On GB300 this kernel takes 41 us for the 1242 x 375, D = 128
-// cost volume against 37.7 us for the CUDA-core kernel, which stays the
-// default (SGM_COST_KERNEL_AUTO).  The matrix products are a small part of
+// Standing.  On GB300 this kernel takes 43.1 us for the 1242 x 375, D = 128
+// cost volume (62-bit codes; 35.2 for D = 60) against 31.3 us (20.5) for the
+// CUDA-core kernel, which stays the default (SGM_COST_KERNEL_AUTO).  The matrix products are a small part of
 // the time: a 128-pixel segment costs about 2800 cycles, most of them moving
 // bytes through shared memory (operand expansion, the cost tile, the record
 // staging, plus the tensor core's and the bulk copy's reads).
@@ -49,8 +49,8 @@
 //   the start differs per pixel), puts each group in the folded
 //   order (two byte permutes) and writes it into the segment's records in a
 //   staging buffer; one cp.async.bulk copies the segment's contiguous records
-//   to the cost volume.  Slots with x - d < 0 or d >= D get nbits, as in the
-//   CUDA-core kernel.
+//   to the cost volume.  Slots with x - d < 0 get nbits and slots d >= D get
+//   kPadCost, as in the CUDA-core kernel.
 //
 // Waits.  The waits are on the mbarriers that MMA completion arrives on; each
 // gives up after about one second.  The CTA then records the timeout in
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     ph = nh;
                 }
             }
-            const bool edge = RAGGED || x < DP - 1;
+            const bool edge = x < DP - 1;
             uint32_t c[2 * CPP];
 #pragma unroll
             for (int m = 0; m < CPP; m++) {
@@ -389,11 +389,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int e = 0; e < 4; e++) {
                         const int dl = 4 * j + e, dh = Dp - 1 - dl;
                         const uint32_t ml = 0xFFu << (8 * (3 - e)), mh = 0xFFu << (8 * e);
-                        if (RAGGED && dl >= D) lo[m] = (lo[m] & ~ml) | (kPadCost << (8 * (3 - e)));
-                        else if (x - dl < 0) lo[m] = (lo[m] & ~ml) | ((uint32_t)nbits << (8 * (3 - e)));
-                        if (RAGGED && dh >= D) hi[m] = (hi[m] & ~mh) | (kPadCost << (8 * e));
-                        else if (x - dh < 0) hi[m] = (hi[m] & ~mh) | ((uint32_t)nbits << (8 * e));
+                        if (x - dl < 0) lo[m] = (lo[m] & ~ml) | ((uint32_t)nbits << (8 * (3 - e)));
+                        if (x - dh < 0) hi[m] = (hi[m] & ~mh) | ((uint32_t)nbits << (8 * e));
                     }
+                }
+                if constexpr (RAGGED) {
+                    // padding: the first Dp - D - 4j bytes of the upper word (D > Dp / 2, so
+                    // the lower one has none); a test of every byte took 46.9 us for 35.2
+                    // at D = 60, 67.8 for 44.5 at D = 100
+                    static_assert(kPadCost == 0xFF, "padding bytes have all bits set");
+                    const int n = min(max(Dp - D - 4 * j, 0), 4);
+                    hi[m] |= n < 4 ? (1u << (8 * n)) - 1u : 0xFFFFFFFFu;
                 }
                 c[2 * m] = __byte_perm(lo[m], hi[m], 0x4532);
                 c[2 * m + 1] = __byte_perm(lo[m], hi[m], 0x6710);
