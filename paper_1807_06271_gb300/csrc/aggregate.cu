@@ -19,8 +19,9 @@
 // directions one after the other read 1.18 GB (the costs are 0.18 GB), 1.37 GB
 // written.  Aggregation in us, directions one after the other -> sweeps: 1242 x 375,
 // D = 128, 8 paths 125 -> 116, 641 x 479, D = 97 90 -> 82, 480 x 752, D = 128 105
-// -> 97, 1920 x 1080, D = 192 1147 -> 1105 (with six pairs per lane), 1280 x 720,
-// D = 64 168 -> 154 (and with the rows between the sweeps 1053 for 1920 x 1080); 640 x 360, D = 60, three of the six directions, 32.8 -> 34.9.
+// -> 97, 1920 x 1080, D = 192 1147 -> 1105 (with six pairs per lane; 1053 with the
+// rows between the sweeps), 1280 x 720, D = 64 168 -> 154; 640 x 360, D = 60, three of
+// the six directions, 32.8 -> 34.9.
 //
 // Arithmetic.  The record of a pixel is folded: pair k holds the disparities
 // (k, Dp-1-k), packed as two 16-bit halves, and a lane holds NP consecutive
@@ -61,7 +62,7 @@
 // by a 1 the compiler cannot see (the job table's unit field), which run on the
 // FMA pipe.
 //
-// Memory.  Costs come through a ring of four stages of 4 to 16 steps per warp in
+// Memory.  Costs come through a ring of four stages of 2 to 16 steps per warp in
 // shared memory, filled by 16-byte asynchronous copies: with loads into registers,
 // 16 steps ahead, a third of the warps' time was waits, as a warp has few
 // scoreboards and a wait for the oldest load also waited for the youngest (1242 x
@@ -233,9 +234,10 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
     return p;
 }
 
-// Job scheduling.  Jobs are numbered long-axis scanlines first, as they take
-// longest.  A warp's first job is its rank: one warp of every SM and scheduler
-// in turn, so that the long-axis jobs spread over all of them.  Later jobs come
+// Job scheduling.  Jobs are numbered in the order of the work list: long-axis
+// scanlines first, as they take longest, or after one sweep from 100 MB of costs
+// on (make_path_jobs).  A warp's first job is its rank: one warp of every SM and
+// scheduler in turn, so that the long-axis jobs spread over all of them.  Later jobs come
 // from one counter, and only when there are more jobs than warps: thousands of
 // warps that start with an atomic on one address pay about 8 ns each, one after
 // the other (320x240, 8 blocks per SM: 61.7 us against 26.3 with 1).

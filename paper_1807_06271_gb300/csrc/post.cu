@@ -11,7 +11,7 @@ namespace {
 // packed maximum order an element of both windows.  The median comes from
 // repeated elimination: of any (k*k + 3)/2 of the elements the smallest and the
 // largest cannot be the median of all, so they are dropped, the next element
-// joins, and so on down to three.  Bound by those minima and maxima (2 x 129
+// joins, and so on down to three.  Bound by those minima and maxima (2 x 132
 // per pixel pair for 5 x 5); a Batcher sort of each pixel's window took 17.3 us on
 // 1280 x 720, this 14.5.  Invalid pixels (0xFF) take part and sort above every
 // valid disparity.
@@ -31,10 +31,10 @@ __device__ __forceinline__ void cmpswap2(uint32_t &a, uint32_t &b) {
 template <int N>
 __device__ __forceinline__ uint32_t median_of(uint32_t (&v)[N]) {
     constexpr int M = (N + 3) / 2;
-    // the set is v[lo .. lo+n-1]; the smallest goes to its front, the largest to its end
+    // the set is v[0 .. n-1]; the smallest goes to its front, the largest to its end
 #pragma unroll
     for (int s = 0; s <= M - 3; s++) {
-        const int n = M - s;  // v[0 .. n-1], where v[n-1] is the element that joined
+        const int n = M - s;  // v[0 .. n-1], where v[0] is the element that joined
 #pragma unroll
         for (int i = 0; i < n / 2; i++) cmpswap2(v[i], v[n - 1 - i]);
 #pragma unroll

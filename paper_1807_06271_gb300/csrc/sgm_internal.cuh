@@ -179,7 +179,8 @@ struct PathJobs {
 };
 
 // Work-queue state of the aggregation kernel: word 0 counts the jobs handed out
-// beyond the warps' first ones (cleared before every launch).
+// beyond the warps' first ones (cleared before every launch).  The rest is not used;
+// the size is part of what sgm.h documents and sgm_scratch_bytes reports.
 constexpr size_t kJobStateBytes = 4224;
 
 // Builds the work list for the directions in `mask`, under the
