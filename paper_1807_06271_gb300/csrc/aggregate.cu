@@ -132,6 +132,10 @@ LaneConfig lane_config(int W, int H, int D, int mask, bool wide, int cpl, bool m
     auto warps = [&](int np_long, int np_other) {
         return lines_long * lanes_of(D, np_long) / 32 + lines_other * lanes_of(D, np_other) / 32;
     };
+    // One pair of 16-bit costs is stored by its index in units of 4 bytes, which must
+    // stay below 2^32 (all other lanes do within the bounds of handle creation): the
+    // columns of an image of 2100 x 65535 alone, say, would go beyond.
+    if (wide && (long long)W * H * __builtin_popcount((unsigned)mask) * Dp / 2 >= (1ll << 32)) return lc;
     if (Dp == 32) {
         if (warps(1, 1) <= 2 * kSchedulers) return {1, 1};
         if (warps(1, 4) <= 3 * kSchedulers) return {1, 4};

@@ -48,9 +48,10 @@ int validate(int W, int H, int D, const sgm_params *p) {
     }
     if (D > kMaxD || W > kMaxW || H > 65535) return SGM_ERR_UNSUPPORTED;
     if (p->median_k > 7) return SGM_ERR_UNSUPPORTED;
-    // kernels index the per-path planes with 32-bit counts of 4 bytes or more (half
-    // of one of these chunks of 8 disparities); the cost ring's index runs up to four
-    // stages of 16 steps of W + 1 pixels past a scanline's end, where nothing is read
+    // kernels index the per-path planes with 32-bit counts of half a chunk of 8
+    // disparities or more (lanes of one pair of 16-bit costs use less, and have a bound
+    // of their own); the cost ring's index runs up to four stages of 16 steps of W + 1
+    // pixels past a scanline's end, where nothing is read
     const long long chunks = ((long long)W * H * npaths + 64ll * (W + 1)) * lanes_per_scanline(D);
     if (chunks >= (1ll << 31)) return SGM_ERR_UNSUPPORTED;
     return SGM_OK;
