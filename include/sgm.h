@@ -286,11 +286,11 @@ int sgm_set_schedule(sgm_handle h, int schedule, int rows_per_cta);
 int sgm_get_schedule(sgm_handle h, int *schedule, int *rows_per_cta);
 
 /* Autotuner: times the pipeline on this pair (device pointers as for
- * sgm_compute; disp is overwritten) with the PLANES schedule at h's own
- * aggregation setting, at the one a new handle of this shape starts with, and at
- * 1, 2, 3, 4 and 6 resident blocks per SM, each with 1, 2 and 4 chunks per lane
- * and the mixed layout where D takes them (sgm_set_aggregation), and, where h
- * can run it, the SWEEP schedule at 2, 4 and 8 rows per block; keeps the fastest for h and for
+ * sgm_compute; disp is overwritten) with the PLANES schedule at 1, 2, 3, 4 and 6
+ * resident aggregation blocks per SM, each with 1, 2 and 4 chunks per lane and the
+ * mixed layout where D takes them (sgm_set_aggregation), at h's own setting and at
+ * the one a new handle of this shape starts with, and, where h can run it, the
+ * SWEEP schedule at 2, 4 and 8 rows per block; keeps the fastest for h and for
  * handles created later in this process with the same W, H, D, path mask,
  * cost, window and P2.  *best_blocks_per_sm (may be NULL) receives the best
  * PLANES setting; sgm_get_schedule tells which schedule won.  Synchronises

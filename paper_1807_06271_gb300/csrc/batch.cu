@@ -185,10 +185,11 @@ extern "C" int sgm_autotune(sgm_handle h, const uint8_t *left, const uint8_t *ri
     const int saved = h->agg_blocks_per_sm, saved_timing = h->timing, saved_cpl = h->agg_cpl;
     const int saved_schedule = h->schedule, saved_rows = h->sweep_rows;
     h->timing = 0;
-    // candidates: h's own setting and what a new handle starts with (1242 x 375, D =
-    // 128, 8 paths starts with 5 blocks, which no other candidate has), then the plane
-    // schedule at each resident-block count and each number of chunks per lane that
-    // runs as such, then the fused sweep at each rows-per-CTA count it can run with
+    // candidates: the plane schedule at each resident-block count and each number of
+    // chunks per lane that runs as such, at h's own setting and at what a new handle
+    // starts with (1242 x 375, D = 128, 8 paths starts with 5 blocks, which no other
+    // candidate has), then the fused sweep at each rows-per-CTA count it can run with.
+    // The last two settings come after the others, as a GPU that was idle is slow at first.
     struct Cand {
         int schedule, param, cpl;
     };
@@ -198,12 +199,12 @@ extern "C" int sgm_autotune(sgm_handle h, const uint8_t *left, const uint8_t *ri
             if (c.param == blocks && c.cpl == cpl) return;
         cands.push_back({SGM_SCHEDULE_PLANES, blocks, cpl});
     };
-    planes(saved, saved_cpl);
-    planes(sgm::default_blocks_per_sm(sgm::make_path_jobs(h->W, h->H, h->D, h->p.path_mask, h->wide != 0, 1)), 1);
     const int cmax = sgm::chunks_apply(h->D, h->wide != 0) ? sgm::chunks_per_lane_max(h->D, h->wide != 0) : 1;
     for (int cpl : {1, 2, sgm::kMixedCpl, 4})
         if ((cpl == sgm::kMixedCpl ? 2 : cpl) <= cmax)
             for (int c : {1, 2, 3, 4, 6}) planes(c, cpl);
+    planes(saved, saved_cpl);
+    planes(sgm::default_blocks_per_sm(sgm::make_path_jobs(h->W, h->H, h->D, h->p.path_mask, h->wide != 0, 1)), 1);
     for (int r : {2, 4, 8})
         if (sgm::sweep_feasible(h, r) == SGM_OK) cands.push_back({SGM_SCHEDULE_SWEEP, r, saved_cpl});
     int best_bps = saved, best_cpl = saved_cpl;
