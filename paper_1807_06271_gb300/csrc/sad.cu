@@ -209,6 +209,8 @@ __global__ void __launch_bounds__(kThreads)
 // 375, D = 128: 85.8, 55.6; 430 x 312, D = 192: 52.1, 32.8.  4 rows took 27.0 / 68.0 /
 // 41.1, segments of 31 pixels 37 / 58.8 / 37.2.
 constexpr int kRows5 = 2, kSegLen = 15;
+// Pixels of a row that a CTA covers.
+__host__ __device__ constexpr int window5_width(int Dp) { return (Dp < 32 ? 32 : 128 / (Dp / 8)) * kSegLen; }
 
 // Whether a W x H image with Dp slots takes this kernel.  With few slots its CTAs are
 // wide, and a small image has too few of them.  Measured, us, the kernel above and
@@ -217,10 +219,12 @@ constexpr int kRows5 = 2, kSegLen = 15;
 //                  1280 x 720 51.4, 47.2, (D = 16) 36.9, 37.0;  640 x 480 (D = 8) 16.5, 18.6
 //   64 slots       320 x 240 14.6, 16.6;  350 x 250 16.5, 16.4;  300 x 300 16.4, 16.4;
 //                  240 x 480 20.6, 16.5;  480 x 260 20.6, 16.7
-//   more           160 x 96 (D = 96) 15.5, 14.1;  100 x 40 (D = 128) 16.4, 13.4
+//   more           160 x 96 (D = 96) 15.5, 14.1;  100 x 40 (D = 128) 16.4, 13.4;  60 x 64 16.5, 13.1
+// An image of a third of a CTA's width leaves most of it idle: 40 x 4000 (D = 128) 49.3,
+// 53.6;  16 x 1000 18.3, 18.8;  but 30 x 400 (D = 200) 22.6, 15.3.
 bool window5_pays(int W, int H, int Dp) {
     const long npx = (long)W * H;
-    return Dp >= 96 || npx >= (Dp == 64 ? 90000 : 400000);
+    return 3 * W > window5_width(Dp) && (Dp >= 96 || npx >= (Dp == 64 ? 90000 : 400000));
 }
 
 template <bool RECT>
@@ -231,7 +235,7 @@ __global__ void __launch_bounds__(128)
     wait_for_predecessor();
     if (job_state && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *job_state = 0u;
     constexpr int S = kRows5 + 4;  // staged rows
-    const int quarters = Dp / 8, segs = Dp < 32 ? 32 : 128 / quarters, width = segs * kSegLen;
+    const int quarters = Dp / 8, width = window5_width(Dp), segs = width / kSegLen;
     const int x0 = blockIdx.x * width, y0 = blockIdx.y * kRows5;
     const int lcols = width + 8, rcols = width + 8 + Dp;
     uint32_t *Lp = reinterpret_cast<uint32_t *>(sad_smem);  // [S][lcols]: (l, l), column x0 - 2 + i
@@ -339,7 +343,7 @@ cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch
         return cudaErrorInvalidValue;
     const int Dp = padded_disparities(D);
     if (ww == 5 && wh == 5 && window5_pays(W, H, Dp)) {
-        const int segs = Dp < 32 ? 32 : 128 / (Dp / 8), width = segs * kSegLen;
+        const int width = window5_width(Dp);
         const size_t smem = (size_t)(kRows5 + 4) * (2 * (width + 8) + Dp) * sizeof(uint32_t);
         return launch_k(maps.lx ? sad5_cost_kernel<true> : sad5_cost_kernel<false>,
                         dim3((W + width - 1) / width, (H + kRows5 - 1) / kRows5), dim3(128), smem, s, left, right, pitch, W, H,
