@@ -209,8 +209,8 @@ __global__ void __launch_bounds__(kThreads)
 // 375, D = 128: 85.8, 55.6; 430 x 312, D = 192: 52.1, 32.8.  4 rows took 27.0 / 68.0 /
 // 41.1, segments of 31 pixels 37 / 58.8 / 37.2.
 constexpr int kRows5 = 2, kSegLen = 15;
-// Pixels of a row that a CTA covers.
-__host__ __device__ constexpr int window5_width(int Dp) { return (Dp < 32 ? 32 : 128 / (Dp / 8)) * kSegLen; }
+// Segments of a row that a CTA covers.
+__host__ __device__ constexpr int window5_segs(int Dp) { return Dp < 32 ? 32 : 128 / (Dp / 8); }
 
 // Whether a W x H image with Dp slots takes this kernel.  With few slots its CTAs are
 // wide, and a small image has too few of them.  Measured, us, the kernel above and
@@ -224,7 +224,7 @@ __host__ __device__ constexpr int window5_width(int Dp) { return (Dp < 32 ? 32 :
 // 53.6;  16 x 1000 18.3, 18.8;  but 30 x 400 (D = 200) 22.6, 15.3.
 bool window5_pays(int W, int H, int Dp) {
     const long npx = (long)W * H;
-    return 3 * W > window5_width(Dp) && (Dp >= 96 || npx >= (Dp == 64 ? 90000 : 400000));
+    return 3 * W > window5_segs(Dp) * kSegLen && (Dp >= 96 || npx >= (Dp == 64 ? 90000 : 400000));
 }
 
 template <bool RECT>
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(128)
     wait_for_predecessor();
     if (job_state && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *job_state = 0u;
     constexpr int S = kRows5 + 4;  // staged rows
-    const int quarters = Dp / 8, width = window5_width(Dp), segs = width / kSegLen;
+    const int quarters = Dp / 8, segs = window5_segs(Dp), width = segs * kSegLen;
     const int x0 = blockIdx.x * width, y0 = blockIdx.y * kRows5;
     const int lcols = width + 8, rcols = width + 8 + Dp;
     uint32_t *Lp = reinterpret_cast<uint32_t *>(sad_smem);  // [S][lcols]: (l, l), column x0 - 2 + i
@@ -343,7 +343,7 @@ cudaError_t launch_sad_cost(const uint8_t *left, const uint8_t *right, int pitch
         return cudaErrorInvalidValue;
     const int Dp = padded_disparities(D);
     if (ww == 5 && wh == 5 && window5_pays(W, H, Dp)) {
-        const int width = window5_width(Dp);
+        const int width = window5_segs(Dp) * kSegLen;
         const size_t smem = (size_t)(kRows5 + 4) * (2 * (width + 8) + Dp) * sizeof(uint32_t);
         return launch_k(maps.lx ? sad5_cost_kernel<true> : sad5_cost_kernel<false>,
                         dim3((W + width - 1) / width, (H + kRows5 - 1) / kRows5), dim3(128), smem, s, left, right, pitch, W, H,
